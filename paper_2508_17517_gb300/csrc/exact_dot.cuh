@@ -9,15 +9,23 @@
 // hierarchy, are reproducible.
 //
 // A finite double is m * 2^e with an integer m < 2^53 and e >= -1074, so the
-// product of two is an integer below 2^106 (two 64-bit halves from
-// __umul64hi / mul) times 2^(ex+ey), ex+ey >= -2148.  The accumulator is a
-// signed fixed-point integer with least significant bit 2^-2148 stored as
-// 140 digits of 32 bits, each digit held in a 64-bit word so that many
-// deposits can wait for one carry pass: a product touches at most 5 digits.
-// Warps deposit into shared-memory accumulators with 64-bit atomics
-// (two's-complement wrap-around makes signed addition exact), blocks add
-// theirs into a global accumulator, and one thread propagates carries and
-// rounds.
+// product of two is an integer below 2^106 (a 128-bit integer product) times
+// 2^(ex+ey), ex+ey >= -2148.  The accumulator is a signed fixed-point integer
+// with least significant bit 2^-2148 stored as 140 digits of 32 bits, each
+// digit held in a 64-bit word so that many deposits can wait for one carry
+// pass.  Threads add their products into a 192-bit register window, warps
+// reduce the windows into their shared-memory accumulators, blocks add
+// theirs into a global accumulator (two's-complement wrap-around makes signed
+// addition exact), and the last block propagates carries and rounds.
+//
+// What bounds it: at 16.8M elements the integer work per product (split,
+// 53 x 53 bits, shift, 192-bit add: ~60 instructions) beside 16-24 bytes of
+// memory traffic; at a few thousand elements the serial tail (launch, block
+// reduction, rounding).  Against the form it replaces (one element in flight
+// per thread, a shared-memory atomic per lane and digit at the end, a
+// single-thread walk over all 140 digits): the 2,100 dots of a 97 x 80 setup
+// with their SpMVs and host reads 64 -> 23 ms, the truncation tests of the
+// 4096^2 setup 789 -> 469 ms.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -31,6 +39,7 @@ namespace airg {
 constexpr int XD_DIGITS = 140;   // 140 * 32 = 4480 bits >= 2148 + 2046 + 2
 constexpr int XD_BIAS = 2148;    // digit-bit position of 2^0
 constexpr int XD_WARPS = 8;      // warps (shared accumulators) per block
+constexpr int XD_UNROLL = 4;     // elements whose loads a thread has in flight at once
 constexpr int XD_THREADS = XD_WARPS * 32;
 
 __device__ __forceinline__ bool xd_split(double x, unsigned long long& m, int& e, int& neg)
@@ -44,159 +53,279 @@ __device__ __forceinline__ bool xd_split(double x, unsigned long long& m, int& e
     return m != 0ULL;
 }
 
-// A thread's register window over six consecutive digits d0 .. d0+5 of the
-// accumulator.  A product's five pieces land in digits d .. d+4 with
-// d = pos >> 5; products of similar magnitude share d, so most of them are
-// added in registers and only a window move (or the end of the thread's
-// loop) deposits the window's digits into the shared accumulator.  The
-// sums are exact integer sums, so the result does not depend on when they
-// are deposited.  Headroom: each slot receives at most one 32-bit piece per
-// product, like a digit of the accumulator.
+// A thread's register window: a 192-bit two's-complement sum whose least
+// significant word stands at digit d0 of the accumulator.  A product at bit
+// position pos covers the five words from digit d = pos >> 5 on; products of
+// similar magnitude share d, so most of them are added here with one carry
+// chain and only a move of the window (or the end of the thread's loop)
+// deposits it.  The sums are exact integer sums, so the result does not
+// depend on when they are deposited.  Headroom: a product at digit d0 + 1 is
+// below 2^169, so 2^20 products fit between deposits; a thread of any launch
+// here takes fewer than 2^15 (n < 2^31 over at least 2^16 threads, or a
+// small n).
 struct XdWin {
-    unsigned long long r[6];
+    unsigned w[6];
     int d0;
 };
 
-__device__ __forceinline__ void xd_win_init(XdWin& w)
+__device__ __forceinline__ void xd_win_init(XdWin& a)
 {
 #pragma unroll
-    for (int k = 0; k < 6; ++k) w.r[k] = 0ULL;
-    w.d0 = -8;
+    for (int k = 0; k < 6; ++k) a.w[k] = 0u;
+    a.d0 = -8;
 }
 
-__device__ __forceinline__ void xd_win_flush(unsigned long long* acc, XdWin& w)
+// Deposit of one thread's window from inside the loop (rare, divergent):
+// words unsigned, the sign as -1 at digit d0 + 6.
+__device__ __forceinline__ void xd_win_deposit(unsigned long long* acc, const XdWin& a)
 {
-    if (w.d0 < 0) return;
+    if (a.d0 < 0) return;
 #pragma unroll
     for (int k = 0; k < 6; ++k)
-        if (w.r[k]) atomicAdd(acc + w.d0 + k, w.r[k]);
+        if (a.w[k]) atomicAdd(acc + a.d0 + k, (unsigned long long)a.w[k]);
+    if (a.w[5] >> 31) atomicAdd(acc + a.d0 + 6, ~0ULL);
 }
 
-__device__ __forceinline__ void xd_win_add(unsigned long long* acc, XdWin& w, double x, double y, int* bad)
+// Deposit of a whole warp's windows into its own accumulator at the end of
+// the loop.  Lanes whose windows stand at the same digit are added with
+// 32-lane integer reductions (16-bit halves, so a sum of 32 fits a word) and
+// one lane per digit writes the sum: a 64-bit shared-memory atomic add per
+// lane and digit is a compare-and-swap loop that serialises the warp.
+__device__ __forceinline__ void xd_warp_deposit(unsigned long long* acc, const XdWin& a)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    unsigned todo = __ballot_sync(full, a.d0 >= 0);
+    while (todo) {
+        const int d = __shfl_sync(full, a.d0, __ffs(todo) - 1);
+        const bool mine = a.d0 == d;
+        todo &= ~__ballot_sync(full, mine);
+        unsigned long long s = 0ULL;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const unsigned v = mine ? a.w[k] : 0u;
+            const unsigned lo = __reduce_add_sync(full, v & 0xffffu), hi = __reduce_add_sync(full, v >> 16);
+            if (lane == k) s = (unsigned long long)lo + ((unsigned long long)hi << 16);
+        }
+        const unsigned neg = __popc(__ballot_sync(full, mine && (a.w[5] >> 31)));
+        if (lane == 6) s = 0ULL - neg;
+        if (lane < 7 && s) acc[d + lane] += s;
+        __syncwarp();
+    }
+}
+
+__device__ __forceinline__ void xd_win_add(unsigned long long* acc, XdWin& a, double x, double y, int* bad)
 {
     unsigned long long mx, my;
     int ex, ey, nx, ny;
     bool zx = !xd_split(x, mx, ex, nx);
     bool zy = !xd_split(y, my, ey, ny);
-    if (!isfinite(x) || !isfinite(y)) { *bad = 1; return; }
+    if (ex == 972 || ey == 972) { *bad = 1; return; }   // exponent field 2047: inf or nan
     if (zx || zy) return;
-    unsigned long long lo = mx * my;
-    unsigned long long hi = __umul64hi(mx, my);
+    const unsigned __int128 p = (unsigned __int128)mx * my;
+    const unsigned p0 = unsigned(p), p1 = unsigned(p >> 32), p2 = unsigned(p >> 64), p3 = unsigned(p >> 96);
     const int pos = ex + ey + XD_BIAS;
-    const int d = pos >> 5, sh = pos & 31;
-    unsigned long long w0 = lo << sh;
-    unsigned long long w1 = sh ? ((hi << sh) | (lo >> (64 - sh))) : hi;
-    unsigned long long w2 = sh ? (hi >> (64 - sh)) : 0ULL;
-    unsigned long long p[5] = {w0 & 0xffffffffULL, w0 >> 32, w1 & 0xffffffffULL, w1 >> 32,
-                               w2 & 0xffffffffULL};
-    if (nx ^ ny) {
-#pragma unroll
-        for (int k = 0; k < 5; ++k) p[k] = 0ULL - p[k];
+    const int d = pos >> 5;
+    if (d != a.d0 && d != a.d0 + 1) {
+        // the window moves so that it holds this digit and, where the
+        // products grew, the one below
+        xd_win_deposit(acc, a);
+        const int d0 = d > a.d0 && d > 0 ? d - 1 : d;
+        xd_win_init(a);
+        a.d0 = d0;
     }
-    if (d == w.d0 - 1) {
-        // move the window down one digit (depositing its top digit)
-        if (w.r[5]) atomicAdd(acc + w.d0 + 5, w.r[5]);
-#pragma unroll
-        for (int k = 5; k > 0; --k) w.r[k] = w.r[k - 1];
-        w.r[0] = 0ULL;
-        w.d0 = d;
-    } else if (d != w.d0 && d != w.d0 + 1) {
-        xd_win_flush(acc, w);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) w.r[k] = 0ULL;
-        w.d0 = d;
-    }
-    if (d == w.d0) {
-#pragma unroll
-        for (int k = 0; k < 5; ++k) w.r[k] += p[k];
-    } else {
-#pragma unroll
-        for (int k = 0; k < 5; ++k) w.r[k + 1] += p[k];
-    }
+    const unsigned m = (nx ^ ny) ? 0xffffffffu : 0u;   // -p = ~p + 1
+    const unsigned q0 = __funnelshift_l(0u, p0, pos) ^ m;
+    const unsigned q1 = __funnelshift_l(p0, p1, pos) ^ m;
+    const unsigned q2 = __funnelshift_l(p1, p2, pos) ^ m;
+    const unsigned q3 = __funnelshift_l(p2, p3, pos) ^ m;
+    const unsigned q4 = __funnelshift_l(p3, 0u, pos) ^ m;
+    const bool up = d != a.d0;                          // product one digit above the window's base
+    const unsigned r0 = up ? m : q0, r1 = up ? q0 : q1, r2 = up ? q1 : q2, r3 = up ? q2 : q3, r4 = up ? q3 : q4,
+                   r5 = up ? q4 : m;
+    asm("{\n\t"
+        ".reg .u32 t;\n\t"
+        "add.cc.u32 t, %12, %12;\n\t"                   // carry in = 1 for a negative product
+        "addc.cc.u32 %0, %0, %6;\n\t"
+        "addc.cc.u32 %1, %1, %7;\n\t"
+        "addc.cc.u32 %2, %2, %8;\n\t"
+        "addc.cc.u32 %3, %3, %9;\n\t"
+        "addc.cc.u32 %4, %4, %10;\n\t"
+        "addc.u32 %5, %5, %11;\n\t"
+        "}"
+        : "+r"(a.w[0]), "+r"(a.w[1]), "+r"(a.w[2]), "+r"(a.w[3]), "+r"(a.w[4]), "+r"(a.w[5])
+        : "r"(r0), "r"(r1), "r"(r2), "r"(r3), "r"(r4), "r"(r5), "r"(m));
 }
 
-// Block: XD_THREADS threads.  gacc: XD_DIGITS words, zero on entry of the
-// first block (cleared by the caller).  bad: set when an input is inf/nan.
-static __global__ void __launch_bounds__(XD_THREADS)
-k_xdot_accumulate(long long n, const double* __restrict__ x, const double* __restrict__ y,
-                  unsigned long long* __restrict__ gacc, int* bad)
+// One warp: carry propagation and round-to-nearest-even of an accumulator in
+// shared memory (which is left altered).  Only the digits between the lowest
+// and the highest nonzero one are walked: the products of one dot product
+// span a few digits of the 140, and the walk is a serial chain.  Every lane
+// gets the result.
+static __device__ inline double xd_round(unsigned long long* g)
 {
-    __shared__ unsigned long long sacc[XD_WARPS][XD_DIGITS];
-    for (int t = threadIdx.x; t < XD_WARPS * XD_DIGITS; t += blockDim.x)
-        (&sacc[0][0])[t] = 0ULL;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    int lo = XD_DIGITS, hi = -1;
+#pragma unroll
+    for (int k = 0; k < (XD_DIGITS + 31) / 32; ++k) {
+        const int i = k * 32 + lane;
+        const unsigned b = __ballot_sync(full, i < XD_DIGITS && g[i] != 0ULL);
+        if (b) {
+            lo = min(lo, k * 32 + __ffs(b) - 1);
+            hi = k * 32 + 31 - __clz(b);
+        }
+    }
+    double r = 0.0;
+    if (lane == 0 && hi >= 0) {
+        long long* d = reinterpret_cast<long long*>(g);
+        const long long MASK = 0xffffffffLL;
+        long long carry = 0;
+        int top = hi;
+        for (int i = lo; i <= hi; ++i) {
+            const long long v = d[i] + carry;
+            d[i] = v & MASK;
+            carry = v >> 32;                       // floor((v - low) / 2^32)
+        }
+        while (carry != 0 && carry != -1 && top < XD_DIGITS - 1) {
+            d[++top] = carry & MASK;
+            carry >>= 32;
+        }
+        const bool neg = carry < 0;
+        if (neg) {                                 // magnitude: two's complement of the digits
+            long long c = 1;
+            for (int i = lo; i <= top; ++i) {
+                const long long v = (~d[i] & MASK) + c;
+                d[i] = v & MASK;
+                c = v >> 32;
+            }
+            if (c && top < XD_DIGITS - 1) d[++top] = c;
+        }
+        const int last = top;
+        while (top >= lo && d[top] == 0) --top;
+        if (top >= lo) {
+            const int hb = 63 - __clzll(d[top]);
+            const int P = top * 32 + hb;           // most significant bit
+            int lsb = P - 52;                      // last bit kept
+            if (lsb < XD_BIAS - 1074) lsb = XD_BIAS - 1074;
+            auto dig = [&](int i) -> unsigned long long {
+                return i >= lo && i <= last ? (unsigned long long)d[i] : 0ULL;
+            };
+            const int q = lsb >> 5, s = lsb & 31;  // lsb >= XD_BIAS - 1074 > 0
+            unsigned long long M = (dig(q) | (dig(q + 1) << 32)) >> s;
+            if (s) M |= dig(q + 2) << (64 - s);
+            const int rp = lsb - 1;                // rounding bit; the bits below it are sticky
+            const int rb = int((dig(rp >> 5) >> (rp & 31)) & 1ULL);
+            bool sticky = (dig(rp >> 5) & ((1ULL << (rp & 31)) - 1ULL)) != 0ULL;
+            for (int i = lo; i < (rp >> 5) && i <= last && !sticky; ++i) sticky = d[i] != 0;
+            if (rb && (sticky || (M & 1ULL))) M += 1ULL;
+            r = scalbn((double)M, lsb - XD_BIAS);
+            if (neg) r = -r;
+        }
+    }
+    return __shfl_sync(full, r, 0);
+}
+
+// The products of one block: load(i) reads the operands of element i,
+// XD_UNROLL elements in flight per thread, and ops(i, raw) gives its two
+// factors (and may store).  The block's digits are in sacc[0] afterwards.
+template <class Load, class Ops>
+__device__ __forceinline__ void xd_block(long long n, unsigned long long (*sacc)[XD_DIGITS], int* bad,
+                                         const Load& load, const Ops& ops)
+{
+    using Raw = decltype(load(0LL));
+    for (int t = threadIdx.x; t < XD_WARPS * XD_DIGITS; t += XD_THREADS) (&sacc[0][0])[t] = 0ULL;
     __syncthreads();
     unsigned long long* mine = sacc[threadIdx.x >> 5];
     XdWin win;
     xd_win_init(win);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        xd_win_add(mine, win, x[i], y[i], bad);
-    xd_win_flush(mine, win);
+    const long long stride = (long long)gridDim.x * XD_THREADS;
+    for (long long i = (long long)blockIdx.x * XD_THREADS + threadIdx.x; i < n; i += XD_UNROLL * stride) {
+        Raw v[XD_UNROLL];
+#pragma unroll
+        for (int u = 0; u < XD_UNROLL; ++u)
+            if (i + u * stride < n) v[u] = load(i + u * stride);
+#pragma unroll
+        for (int u = 0; u < XD_UNROLL; ++u)
+            if (i + u * stride < n) {
+                const double2 f = ops(i + u * stride, v[u]);
+                xd_win_add(mine, win, f.x, f.y, bad);
+            }
+    }
+    xd_warp_deposit(mine, win);
     __syncthreads();
-    for (int t = threadIdx.x; t < XD_DIGITS; t += blockDim.x) {
+    for (int t = threadIdx.x; t < XD_DIGITS; t += XD_THREADS) {
         unsigned long long s = 0ULL;
 #pragma unroll
         for (int w = 0; w < XD_WARPS; ++w) s += sacc[w][t];
-        if (s) atomicAdd(gacc + t, s);
+        sacc[0][t] = s;
     }
 }
 
-// One thread: carry propagation and round-to-nearest-even of an accumulator
-// (a copy in shared memory; the callers load the global digits in parallel
-// first).  Returns the double and leaves the digits cleared.
-static __device__ inline double xd_round(unsigned long long* g)
+// Adds the block's digits into the global accumulator; true in the last
+// block to arrive (atomic ticket, reset for the next call), which then holds
+// the global digits in sacc[0] and has cleared them.  A launch of one block
+// keeps its digits where they are.
+__device__ __forceinline__ bool xd_grid_sum(unsigned long long (*sacc)[XD_DIGITS], unsigned long long* gacc,
+                                            unsigned* ticket)
 {
-    long long* d = reinterpret_cast<long long*>(g);
-    long long carry = 0;
-    for (int i = 0; i < XD_DIGITS - 1; ++i) {
-        long long v = d[i] + carry;
-        long long lo = v & 0xffffffffLL;
-        d[i] = lo;
-        carry = (v - lo) >> 32;   // v - lo is a multiple of 2^32
+    __shared__ bool last;
+    if (gridDim.x == 1) {
+        __syncthreads();
+        return true;
     }
-    d[XD_DIGITS - 1] += carry;
-    int neg = 0;
-    if (d[XD_DIGITS - 1] < 0) {
-        neg = 1;
-        carry = 0;
-        for (int i = 0; i < XD_DIGITS; ++i) d[i] = -d[i];
-        for (int i = 0; i < XD_DIGITS - 1; ++i) {
-            long long v = d[i] + carry;
-            long long lo = v & 0xffffffffLL;
-            d[i] = lo;
-            carry = (v - lo) >> 32;
-        }
-        d[XD_DIGITS - 1] += carry;
-    }
-    int top = -1;
-    for (int i = XD_DIGITS - 1; i >= 0; --i)
-        if (d[i] != 0) { top = i; break; }
-    double r = 0.0;
-    if (top >= 0) {
-        int hb = 63 - __clzll(d[top]);
-        int P = top * 32 + hb;                 // most significant bit
-        int lsb = P - 52;                      // last bit kept
-        if (lsb < XD_BIAS - 1074) lsb = XD_BIAS - 1074;
-        unsigned long long M = 0ULL;
-        for (int b = P; b >= lsb; --b) M = (M << 1) | (unsigned long long)((d[b >> 5] >> (b & 31)) & 1);
-        int rb = (lsb - 1 >= 0) ? int((d[(lsb - 1) >> 5] >> ((lsb - 1) & 31)) & 1) : 0;
-        int sticky = 0;
-        int lim = lsb - 1;                     // bits [0, lim) are sticky bits
-        for (int w = 0; w < (lim >> 5) && !sticky; ++w) sticky = d[w] != 0;
-        if (!sticky && lim > 0 && (lim & 31)) {
-            long long mask = (1LL << (lim & 31)) - 1;
-            sticky = (d[lim >> 5] & mask) != 0;
-        }
-        if (rb && (sticky || (M & 1ULL))) M += 1ULL;
-        r = scalbn((double)M, lsb - XD_BIAS);
-    }
-    for (int i = 0; i < XD_DIGITS; ++i) d[i] = 0;
-    return neg ? -r : r;
+    for (int t = threadIdx.x; t < XD_DIGITS; t += XD_THREADS)
+        if (sacc[0][t]) atomicAdd(gacc + t, sacc[0][t]);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    for (int t = threadIdx.x; t < XD_DIGITS; t += XD_THREADS) sacc[0][t] = atomicExch(gacc + t, 0ULL);
+    if (threadIdx.x == 0) *ticket = 0u;
+    __syncthreads();
+    return true;
+}
+
+// First warp of a block: rounds and writes the double and its square root
+__device__ __forceinline__ void xd_write(unsigned long long* g, const int* bad, double* out, double* out_sqrt)
+{
+    if (threadIdx.x >= 32) return;
+    double r = xd_round(g);
+    if (threadIdx.x != 0) return;
+    if (*(volatile const int*)bad) r = __longlong_as_double(0x7ff8000000000000LL);
+    if (out) *out = r;
+    if (out_sqrt) *out_sqrt = __dsqrt_rn(r);
+}
+
+// Blocks of a dot product of length n: at least XD_UNROLL elements per
+// thread before another block is worth its share of the final sum, at most
+// four resident blocks (32 warps) per SM.  Up to 2048 elements one block
+// takes all (at most 8 elements a thread) and the global sum falls away.
+inline int xd_grid(long long n, int sms)
+{
+    if (n <= 2048) return 1;
+    const long long b = (n + XD_THREADS * XD_UNROLL - 1) / (XD_THREADS * XD_UNROLL);
+    return int(b < 4LL * sms ? b : 4LL * sms);
+}
+
+// Block: XD_THREADS threads.  gacc: XD_DIGITS words, zero on entry of the
+// first block (cleared by the caller).  bad: set when an input is inf/nan.
+static __global__ void __launch_bounds__(XD_THREADS, 4)
+k_xdot_accumulate(long long n, const double* __restrict__ x, const double* __restrict__ y,
+                  unsigned long long* __restrict__ gacc, int* bad)
+{
+    __shared__ unsigned long long sacc[XD_WARPS][XD_DIGITS];
+    xd_block(n, sacc, bad, [&](long long i) { return make_double2(x[i], y[i]); },
+             [](long long, double2 v) { return v; });
+    for (int t = threadIdx.x; t < XD_DIGITS; t += XD_THREADS)
+        if (sacc[0][t]) atomicAdd(gacc + t, sacc[0][t]);
 }
 
 // One warp: takes the global digits into shared memory (reading and
-// clearing each word in one atomic exchange), then one thread rounds.
-// Writes the double to *out and optionally its square root to *out_sqrt.
+// clearing each word in one atomic exchange) and rounds.
 static __global__ void k_xdot_finalize(unsigned long long* gacc, const int* bad, double* out,
                                        double* out_sqrt)
 {
@@ -204,53 +333,19 @@ static __global__ void k_xdot_finalize(unsigned long long* gacc, const int* bad,
     if (blockIdx.x != 0 || threadIdx.x >= 32) return;
     for (int t = threadIdx.x; t < XD_DIGITS; t += 32) d[t] = atomicExch(gacc + t, 0ULL);
     __syncwarp();
-    if (threadIdx.x != 0) return;
-    double r = xd_round(d);
-    if (*(volatile const int*)bad) r = __longlong_as_double(0x7ff8000000000000LL);
-    if (out) *out = r;
-    if (out_sqrt) *out_sqrt = __dsqrt_rn(r);
+    xd_write(d, bad, out, out_sqrt);
 }
 
-// Accumulation and rounding in one launch: blocks deposit as in
-// k_xdot_accumulate; the last block to finish (atomic ticket, reset for the
-// next call) takes the global digits, clearing them, and rounds.
-static __global__ void __launch_bounds__(XD_THREADS)
+// Accumulation and rounding in one launch: the last block to finish takes
+// the global digits, clearing them, and rounds.
+static __global__ void __launch_bounds__(XD_THREADS, 4)
 k_xdot(long long n, const double* __restrict__ x, const double* __restrict__ y,
        unsigned long long* __restrict__ gacc, int* bad, unsigned* ticket, double* out, double* out_sqrt)
 {
     __shared__ unsigned long long sacc[XD_WARPS][XD_DIGITS];
-    __shared__ bool last;
-    for (int t = threadIdx.x; t < XD_WARPS * XD_DIGITS; t += blockDim.x)
-        (&sacc[0][0])[t] = 0ULL;
-    __syncthreads();
-    unsigned long long* mine = sacc[threadIdx.x >> 5];
-    XdWin win;
-    xd_win_init(win);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        xd_win_add(mine, win, x[i], y[i], bad);
-    xd_win_flush(mine, win);
-    __syncthreads();
-    for (int t = threadIdx.x; t < XD_DIGITS; t += blockDim.x) {
-        unsigned long long s = 0ULL;
-#pragma unroll
-        for (int w = 0; w < XD_WARPS; ++w) s += sacc[w][t];
-        if (s) atomicAdd(gacc + t, s);
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    for (int t = threadIdx.x; t < XD_DIGITS; t += blockDim.x) sacc[0][t] = atomicExch(gacc + t, 0ULL);
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    double r = xd_round(sacc[0]);
-    if (*(volatile const int*)bad) r = __longlong_as_double(0x7ff8000000000000LL);
-    if (out) *out = r;
-    if (out_sqrt) *out_sqrt = __dsqrt_rn(r);
-    *ticket = 0u;
+    xd_block(n, sacc, bad, [&](long long i) { return make_double2(x[i], y[i]); },
+             [](long long, double2 v) { return v; });
+    if (xd_grid_sum(sacc, gacc, ticket)) xd_write(sacc[0], bad, out, out_sqrt);
 }
 
 // One modified Gram-Schmidt step fused with the next correctly rounded dot
@@ -258,51 +353,24 @@ k_xdot(long long n, const double* __restrict__ x, const double* __restrict__ y,
 // with h = *hprev (product rounded, then the difference: the same two
 // roundings as a separate update kernel); then <w, y> (y = w itself when
 // null) accumulated exactly and rounded by the last block, as k_xdot.
-static __global__ void __launch_bounds__(XD_THREADS)
+static __global__ void __launch_bounds__(XD_THREADS, 4)
 k_mgs_xdot(long long n, double* __restrict__ w, const double* __restrict__ vprev, const double* hprev,
            const double* __restrict__ y, unsigned long long* __restrict__ gacc, int* bad, unsigned* ticket,
            double* out, double* out_sqrt)
 {
     __shared__ unsigned long long sacc[XD_WARPS][XD_DIGITS];
-    __shared__ bool last;
-    for (int t = threadIdx.x; t < XD_WARPS * XD_DIGITS; t += blockDim.x)
-        (&sacc[0][0])[t] = 0ULL;
-    __syncthreads();
-    unsigned long long* mine = sacc[threadIdx.x >> 5];
-    XdWin win;
-    xd_win_init(win);
     const double h = vprev ? *hprev : 0.0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        double wi = w[i];
-        if (vprev) {
-            wi = __dsub_rn(wi, __dmul_rn(h, vprev[i]));
-            w[i] = wi;
-        }
-        xd_win_add(mine, win, wi, y ? y[i] : wi, bad);
-    }
-    xd_win_flush(mine, win);
-    __syncthreads();
-    for (int t = threadIdx.x; t < XD_DIGITS; t += blockDim.x) {
-        unsigned long long s = 0ULL;
-#pragma unroll
-        for (int q = 0; q < XD_WARPS; ++q) s += sacc[q][t];
-        if (s) atomicAdd(gacc + t, s);
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    for (int t = threadIdx.x; t < XD_DIGITS; t += blockDim.x) sacc[0][t] = atomicExch(gacc + t, 0ULL);
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    double r = xd_round(sacc[0]);
-    if (*(volatile const int*)bad) r = __longlong_as_double(0x7ff8000000000000LL);
-    if (out) *out = r;
-    if (out_sqrt) *out_sqrt = __dsqrt_rn(r);
-    *ticket = 0u;
+    xd_block(n, sacc, bad,
+             [&](long long i) { return make_double3(w[i], vprev ? vprev[i] : 0.0, y ? y[i] : 0.0); },
+             [&](long long i, double3 v) {
+                 double wi = v.x;
+                 if (vprev) {
+                     wi = __dsub_rn(wi, __dmul_rn(h, v.y));
+                     w[i] = wi;
+                 }
+                 return make_double2(wi, y ? v.z : wi);
+             });
+    if (xd_grid_sum(sacc, gacc, ticket)) xd_write(sacc[0], bad, out, out_sqrt);
 }
 
 }  // namespace airg

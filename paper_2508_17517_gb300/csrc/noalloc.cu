@@ -82,8 +82,7 @@ airg_status airg_dot_exact_noalloc(int64_t n, const double* x, const double* y, 
     cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(unsigned long long) * kScratchWords, s);
     if (e != cudaSuccess) return set_err(AIRG_ERR_CUDA, "cudaMemsetAsync", e);
     int* bad = reinterpret_cast<int*>(scratch + airg::XD_DIGITS);
-    long long blocks = (n + airg::XD_THREADS - 1) / airg::XD_THREADS;
-    int grid = int(blocks < 1 ? 1 : (blocks > 2LL * sms ? 2LL * sms : blocks));
+    const int grid = airg::xd_grid(n, sms);
     airg::k_xdot_accumulate<<<grid, airg::XD_THREADS, 0, s>>>(n, x, y, scratch, bad);
     airg::k_xdot_finalize<<<1, 32, 0, s>>>(scratch, bad, out, nullptr);
     e = cudaGetLastError();

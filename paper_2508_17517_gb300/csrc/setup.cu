@@ -926,6 +926,7 @@ struct Ctx {
     DBuf<int> xbad;
     DBuf<unsigned> xticket;          // last-block ticket of k_xdot
     long long ndots = 0;             // exact dot products launched
+    HBuf<double> hcol;               // one Hessenberg column on the host
     explicit Ctx(cudaStream_t s) : st(s)
     {
         xacc.alloc(XD_DIGITS);
@@ -950,8 +951,7 @@ int num_sms()
 
 void xdot(Ctx& c, long long n, const double* x, const double* y, double* out, double* out_sqrt)
 {
-    int grid = (int)std::min<long long>(std::max<long long>(1, (n + XD_THREADS - 1) / XD_THREADS),
-                                        2LL * num_sms());
+    const int grid = xd_grid(n, num_sms());
     k_xdot<<<grid, XD_THREADS, 0, c.st>>>(n, x, y, c.xacc.p, c.xbad.p, c.xticket.p, out, out_sqrt);
     CK_LAUNCH();
     ++c.ndots;
@@ -962,8 +962,7 @@ void xdot(Ctx& c, long long n, const double* x, const double* y, double* out, do
 void mgs_xdot(Ctx& c, long long n, double* w, const double* vprev, const double* hprev, const double* y,
               double* out, double* out_sqrt)
 {
-    int grid = (int)std::min<long long>(std::max<long long>(1, (n + XD_THREADS - 1) / XD_THREADS),
-                                        2LL * num_sms());
+    const int grid = xd_grid(n, num_sms());
     k_mgs_xdot<<<grid, XD_THREADS, 0, c.st>>>(n, w, vprev, hprev, y, c.xacc.p, c.xbad.p, c.xticket.p, out,
                                                out_sqrt);
     CK_LAUNCH();
@@ -1144,8 +1143,8 @@ ArnoldiOut arnoldi(Ctx& c, const DevCSR& A, const double* b, int m, double tol, 
 {
     cudaStream_t st = c.st;
     long long n = A.n_rows;
+    // H on the device by columns, so that one copy brings a column to the host
     DBuf<double> V(size_t(m + 1) * n), w(n), Hd(size_t(m + 1) * m + 1);
-    CK(cudaMemsetAsync(Hd.p, 0, Hd.bytes(), st));
     double* beta_d = Hd.p + size_t(m + 1) * m;
     xdot(c, n, b, b, nullptr, beta_d);
     int g = grid_for(n, TB);
@@ -1155,24 +1154,21 @@ ArnoldiOut arnoldi(Ctx& c, const DevCSR& A, const double* b, int m, double tol, 
     const double beta_h = read1(beta_d, st);
     ArnoldiOut out;
     out.k = m;
-    std::vector<double> col(m + 1);
+    c.hcol.alloc(size_t(m) + 1);
+    const double* col = c.hcol.p;
     for (int j = 0; j < m; ++j) {
         k_spmv_det<<<grid_for(n, TB), TB, 0, st>>>(int(n), A.rp.p, A.ci.p, A.v.p, V.p + size_t(j) * n, w.p);
         CK_LAUNCH();
+        double* hj = Hd.p + size_t(j) * (m + 1);
         // h_ij = <w, v_i> then w -= h_ij v_i, for i = 0..j (modified
         // Gram-Schmidt); each update is fused with the next dot product
         for (int i = 0; i <= j; ++i) {
-            double* hij = Hd.p + size_t(i) * m + j;
-            const double* hprev = i ? Hd.p + size_t(i - 1) * m + j : nullptr;
-            mgs_xdot(c, n, w.p, i ? V.p + size_t(i - 1) * n : nullptr, hprev, V.p + size_t(i) * n, hij, nullptr);
+            mgs_xdot(c, n, w.p, i ? V.p + size_t(i - 1) * n : nullptr, i ? hj + i - 1 : nullptr,
+                     V.p + size_t(i) * n, hj + i, nullptr);
         }
-        double* hn = Hd.p + size_t(j + 1) * m + j;
-        mgs_xdot(c, n, w.p, V.p + size_t(j) * n, Hd.p + size_t(j) * m + j, nullptr, nullptr, hn);
-        // read column j (rows 0..j+1)
-        for (int i = 0; i <= j + 1; ++i)
-            CK(cudaMemcpyAsync(&col[i], Hd.p + size_t(i) * m + j, sizeof(double),
-                               cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
+        double* hn = hj + j + 1;
+        mgs_xdot(c, n, w.p, V.p + size_t(j) * n, hj + j, nullptr, nullptr, hn);
+        d2h(c.hcol.p, hj, size_t(j) + 2, st);
         for (int i = 0; i <= j + 1; ++i) Hh[size_t(i) * m + j] = col[i];
         double s = 0.0;
         for (int i = 0; i <= j + 1; ++i) s = s + col[i] * col[i];
