@@ -31,42 +31,106 @@ constexpr int MAXB = 16;         // restart length of the batched FGMRES
 constexpr int MAXK = 128;        // right-hand sides per batch (KW <= 4)
 
 
-// Rows of operator S times the k right-hand sides x ([row][rhs]): row r is
-// handled by PW warps of a block (BT/32/PW rows per block), lanes over the
-// right-hand sides (q = lane + 32 j, j < KW).  Warp `part` of a row adds the
-// row's stored entries e = part, part + PW, ... in order (after the dense
-// diagonal term, part 0); with PW > 1 the partial rows meet in shared memory
-// and are added in part order.  PW is fixed per operator from its row
-// lengths (1 for short rows, 4 for long ones), so results do not depend on
-// timing.  pre(r, lane) loads the row's other operands before the product,
-// so those loads overlap the gathers; entries are taken four at a time with
-// all their loads issued before their FMAs, which run in entry order.  Then
-// epi(r, lane, acc, pre) runs once per row.  `dot` = false skips the product
-// (acc = 0).  Every thread of the block reaches the barrier.
-template <class T, int KW, int PW, class V, class Pre, class Epi>
-__device__ __forceinline__ void bfor_rows(const SellView<T, V>& S, const T* __restrict__ x, int k, bool dot,
-                                          const Pre& pre, const Epi& epi, int rev = 0)
+// How the lanes of a warp share the k right-hand sides of a row: each lane
+// holds VEC adjacent ones (one 16-byte load where k allows it, else one), a
+// group of 2^lg lanes covers a row, and the warp's other groups take the
+// next rows.  A lane then keeps the loads of 32 >> lg rows' worth of work in
+// flight per warp instruction, and a narrow batch leaves no lane idle: with
+// one warp per row, 7 right-hand sides used 7 of 32 lanes of every FP64
+// instruction, and a row of 2-3 entries was a warp's whole work.  Wider
+// batches than a warp covers take KW steps of it.  The sums of a (row,
+// right-hand side) are the same in every shape.
+// Bound: FP64 issue and gather latency on the long rows, memory on the short
+// ones.  Measured before and after, per launch: coarse step of 7 right-hand
+// sides (10k rows of 71 entries, FP64) 55.6 -> 20.2 us; of 32 (41k rows of
+// 199 entries, FP32) 197 -> 81 us; first smoother term of 32 (1.8M rows of
+// 1.4 entries) 335 -> 174 us (4.3 TB/s); FP64 top-level product of 32 (4.2M
+// rows of 3 entries) 1.64 -> 1.15 ms.
+template <class T, int VEC, int KW>
+struct Lanes {
+    int ql, lg, k;
+    __device__ __forceinline__ int q(int j) const { return (ql + (j << lg)) * VEC; }
+    __device__ __forceinline__ bool ok(int j) const { return q(j) < k; }
+};
+template <class T, int VEC>
+struct alignas(sizeof(T) * VEC) Pack {
+    T v[VEC];
+};
+// this lane's values of one row
+template <class T, int VEC, int KW>
+struct Vals {
+    Pack<T, VEC> p[KW];
+};
+
+template <class T, int VEC, int KW>
+__device__ __forceinline__ Vals<T, VEC, KW> bload(const Lanes<T, VEC, KW>& L, const T* __restrict__ a, long long r)
 {
-    using PV = decltype(pre(0, 0));
+    Vals<T, VEC, KW> o;
+#pragma unroll
+    for (int j = 0; j < KW; ++j) {
+        if (a && r >= 0 && L.ok(j)) o.p[j] = *reinterpret_cast<const Pack<T, VEC>*>(a + size_t(r) * L.k + L.q(j));
+        else
+#pragma unroll
+            for (int u = 0; u < VEC; ++u) o.p[j].v[u] = T(0);
+    }
+    return o;
+}
+template <class T, int VEC, int KW>
+__device__ __forceinline__ void bstore(const Lanes<T, VEC, KW>& L, T* a, long long r, const Vals<T, VEC, KW>& o)
+{
+#pragma unroll
+    for (int j = 0; j < KW; ++j)
+        if (L.ok(j)) *reinterpret_cast<Pack<T, VEC>*>(a + size_t(r) * L.k + L.q(j)) = o.p[j];
+}
+// o = f(values of the operands), element by element
+template <class T, int VEC, int KW, class F, class... A>
+__device__ __forceinline__ Vals<T, VEC, KW> beach(const F& f, const Vals<T, VEC, KW>& a, const A&... more)
+{
+    Vals<T, VEC, KW> o;
+#pragma unroll
+    for (int j = 0; j < KW; ++j)
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) o.p[j].v[u] = f(a.p[j].v[u], more.p[j].v[u]...);
+    return o;
+}
+
+// Rows of operator S times the k right-hand sides x ([row][rhs]): row r is
+// handled by one lane group (above) of PW warps of a block.  Warp `part` of
+// a row adds the row's stored entries e = part, part + PW, ... in order
+// (after the dense diagonal term, part 0); with PW > 1 the partial rows meet
+// in shared memory and are added in part order.  PW is fixed per operator
+// from its row lengths (1 for short rows, 4 for long ones), so results do
+// not depend on timing.  pre(r, L) loads the row's other operands before the
+// product, so those loads overlap the gathers; entries are taken four at a
+// time with all their loads issued before their FMAs, which run in entry
+// order.  Then epi(r, L, sums, pre) runs once per row.  `dot` = false skips
+// the product (sums 0).  Every thread of the block reaches the barrier.
+template <class T, int VEC, int KW, int PW, class V, class Pre, class Epi>
+__device__ __forceinline__ void bfor_rows(const SellView<T, V>& S, const T* __restrict__ x, int k, int lg,
+                                          bool dot, const Pre& pre, const Epi& epi, int rev = 0)
+{
+    using LN = Lanes<T, VEC, KW>;
+    using PK = Pack<T, VEC>;
+    using PV = decltype(pre(0, LN{}));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int part = warp % PW;
+    const LN L{lane & ((1 << lg) - 1), lg, k};
     // rev != 0: blocks take the rows in reverse order (serpentine chains)
     const int bx = rev ? int(gridDim.x) - 1 - int(blockIdx.x) : int(blockIdx.x);
-    const int r = bx * (BT / 32 / PW) + warp / PW;
-    const bool valid = r < S.n_rows;
+    const long long rr = ((long long)bx * (BT / 32 / PW) + warp / PW) * (32 >> lg) + (lane >> lg);
+    const bool valid = rr < S.n_rows;
+    const int r = valid ? int(rr) : 0;
     const bool lead = valid && part == 0;
-    const PV pv = lead ? pre(r, lane) : PV{};
-    T acc[KW];
+    const PV pv = lead ? pre(r, L) : PV{};
+    Vals<T, VEC, KW> acc;
 #pragma unroll
-    for (int j = 0; j < KW; ++j) acc[j] = T(0);
+    for (int j = 0; j < KW; ++j)
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) acc.p[j].v[u] = T(0);
     if (valid && dot) {
         if (part == 0 && S.diag) {
             const T dg = __ldg(S.diag + r);
-#pragma unroll
-            for (int j = 0; j < KW; ++j) {
-                int q = lane + 32 * j;
-                if (q < k) acc[j] = dg * x[size_t(r) * k + q];
-            }
+            acc = beach<T, VEC, KW>([&](T xv) { return dg * xv; }, bload(L, x, r));
         }
         const int s = r >> 5;
         const int b = S.sptr[s] + (r & 31), w = (S.sptr[s + 1] - S.sptr[s]) >> 5;
@@ -80,161 +144,155 @@ __device__ __forceinline__ void bfor_rows(const SellView<T, V>& S, const T* __re
                 v[u] = ldval<T>(S.val + idx);
                 xr[u] = x + size_t(__ldg(S.col + idx)) * k;
             }
-            T xv[4][KW];
+            PK xv[4][KW];
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int j = 0; j < KW; ++j) {
-                    int q = lane + 32 * j;
-                    xv[u][j] = q < k ? xr[u][q] : T(0);
+                for (int j = 0; j < KW; ++j)
+                    if (L.ok(j)) xv[u][j] = *reinterpret_cast<const PK*>(xr[u] + L.q(j));
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int j = 0; j < KW; ++j)
+                    if (L.ok(j))
+#pragma unroll
+                        for (int i = 0; i < VEC; ++i) acc.p[j].v[i] = fma(v[u], xv[u][j].v[i], acc.p[j].v[i]);
+        }
+        if (e < w) {   // up to three entries left, their loads together too
+            T v[3];
+            const T* xr[3];
+            PK xv[3][KW];
+#pragma unroll
+            for (int u = 0; u < 3; ++u)
+                if (e + u * PW < w) {
+                    const int idx = b + 32 * (e + u * PW);
+                    v[u] = ldval<T>(S.val + idx);
+                    xr[u] = x + size_t(__ldg(S.col + idx)) * k;
                 }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < 3; ++u)
 #pragma unroll
-                for (int j = 0; j < KW; ++j) acc[j] = fma(v[u], xv[u][j], acc[j]);
-        }
-        for (; e < w; e += PW) {
-            const int idx = b + 32 * e;
-            const T v = ldval<T>(S.val + idx);
-            const T* xr = x + size_t(__ldg(S.col + idx)) * k;
+                for (int j = 0; j < KW; ++j)
+                    if (e + u * PW < w && L.ok(j)) xv[u][j] = *reinterpret_cast<const PK*>(xr[u] + L.q(j));
 #pragma unroll
-            for (int j = 0; j < KW; ++j) {
-                int q = lane + 32 * j;
-                if (q < k) acc[j] = fma(v, xr[q], acc[j]);
-            }
+            for (int u = 0; u < 3; ++u)
+#pragma unroll
+                for (int j = 0; j < KW; ++j)
+                    if (e + u * PW < w && L.ok(j))
+#pragma unroll
+                        for (int i = 0; i < VEC; ++i) acc.p[j].v[i] = fma(v[u], xv[u][j].v[i], acc.p[j].v[i]);
         }
     }
     if constexpr (PW > 1) {
-        __shared__ T red[BT / 32][KW * 32];
+        __shared__ T red[BT / 32][KW * VEC][32];
 #pragma unroll
-        for (int j = 0; j < KW; ++j) red[warp][j * 32 + lane] = acc[j];
+        for (int j = 0; j < KW; ++j)
+#pragma unroll
+            for (int u = 0; u < VEC; ++u) red[warp][j * VEC + u][lane] = acc.p[j].v[u];
         __syncthreads();
         if (part == 0) {
 #pragma unroll
             for (int p = 1; p < PW; ++p)
 #pragma unroll
-                for (int j = 0; j < KW; ++j) acc[j] += red[warp + p][j * 32 + lane];
+                for (int j = 0; j < KW; ++j)
+#pragma unroll
+                    for (int u = 0; u < VEC; ++u) acc.p[j].v[u] += red[warp + p][j * VEC + u][lane];
         }
     }
-    if (lead) epi(r, lane, acc, pv);
+    if (lead) epi(r, L, acc, pv);
 }
 
-// this lane's values of row r of v ([row][rhs]); b: a second vector
-template <class T, int KW>
-struct RowVals {
-    T a[KW], b[KW];
+// blocks for n rows at PW warps per lane group of 2^lg lanes
+inline int grid_rows(long long n, int pw, int lg)
+{
+    const int per = (BT / 32 / pw) * (32 >> lg);
+    return grid_for(n, per);
+}
+
+template <class T, int VEC, int KW>
+struct Vals2 {
+    Vals<T, VEC, KW> a, b;
 };
-template <class T, int KW>
-__device__ __forceinline__ RowVals<T, KW> row_vals(const T* __restrict__ va, const T* __restrict__ vb,
-                                                   long long ra, long long rb, int lane, int k)
+
+template <class T, int VEC, int KW, int PW>
+__global__ void kb_spmv(SellView<T> S, const T* __restrict__ x, T* __restrict__ y, int k, int lg)
 {
-    RowVals<T, KW> o;
-#pragma unroll
-    for (int j = 0; j < KW; ++j) {
-        int q = lane + 32 * j;
-        o.a[j] = (va && q < k) ? va[size_t(ra) * k + q] : T(0);
-        o.b[j] = (vb && rb >= 0 && q < k) ? vb[size_t(rb) * k + q] : T(0);
-    }
-    return o;
+    using LN = Lanes<T, VEC, KW>;
+    using VL = Vals<T, VEC, KW>;
+    bfor_rows<T, VEC, KW, PW>(S, x, k, lg, true, [](int, const LN&) { return 0; },
+                              [&](int r, const LN& L, const VL& d, int) { bstore(L, y, r, d); });
 }
 
-// blocks for n rows at PW warps per row
-inline int grid_rows(long long n, int pw) { return grid_for(n * pw, BT / 32); }
-
-template <class T, int KW, int PW>
-__global__ void kb_spmv(SellView<T> S, const T* __restrict__ x, T* __restrict__ y, int k)
-{
-    bfor_rows<T, KW, PW>(S, x, k, true, [](int, int) { return 0; }, [&](int r, int lane, const T (&a)[KW], int) {
-#pragma unroll
-        for (int j = 0; j < KW; ++j) {
-            int q = lane + 32 * j;
-            if (q < k) y[size_t(r) * k + q] = a[j];
-        }
-    });
-}
-
-template <class T, int KW, int PW, class V = T>
+template <class T, int VEC, int KW, int PW, class V = T>
 __global__ void kb_restrict(SellView<T, V> Z, const T* __restrict__ sf, const T* __restrict__ sc,
-                            T* __restrict__ dc, int k)
+                            T* __restrict__ dc, int k, int lg)
 {
-    bfor_rows<T, KW, PW>(Z, sf, k, true,
-                         [&](int r, int lane) { return row_vals<T, KW>(sc, nullptr, r, -1, lane, k); },
-                         [&](int r, int lane, const T (&a)[KW], const RowVals<T, KW>& pv) {
-#pragma unroll
-        for (int j = 0; j < KW; ++j) {
-            int q = lane + 32 * j;
-            if (q < k) dc[size_t(r) * k + q] = pv.a[j] + a[j];
-        }
-    });
+    using LN = Lanes<T, VEC, KW>;
+    using VL = Vals<T, VEC, KW>;
+    bfor_rows<T, VEC, KW, PW>(Z, sf, k, lg, true, [&](int r, const LN& L) { return bload(L, sc, r); },
+                              [&](int r, const LN& L, const VL& d, const VL& c) {
+                                  bstore(L, dc, r, beach<T, VEC, KW>([](T a, T b) { return a + b; }, c, d));
+                              });
 }
 
-template <class T, int KW, int PW>
+template <class T, int VEC, int KW, int PW>
 __global__ void kb_fresid(SellView<T> M, const T* __restrict__ rf, const T* __restrict__ ec,
-                          T* __restrict__ t, T* __restrict__ w, T ap, int k)
+                          T* __restrict__ t, T* __restrict__ w, T ap, int k, int lg)
 {
-    bfor_rows<T, KW, PW>(M, ec, k, true,
-                         [&](int r, int lane) { return row_vals<T, KW>(rf, nullptr, r, -1, lane, k); },
-                         [&](int r, int lane, const T (&a)[KW], const RowVals<T, KW>& pv) {
-#pragma unroll
-        for (int j = 0; j < KW; ++j) {
-            int q = lane + 32 * j;
-            if (q < k) {
-                size_t o = size_t(r) * k + q;
-                T tt = pv.a[j] - a[j];
-                t[o] = tt;
-                w[o] = ap * tt;
-            }
-        }
-    });
+    using LN = Lanes<T, VEC, KW>;
+    using VL = Vals<T, VEC, KW>;
+    bfor_rows<T, VEC, KW, PW>(M, ec, k, lg, true, [&](int r, const LN& L) { return bload(L, rf, r); },
+                              [&](int r, const LN& L, const VL& d, const VL& f) {
+                                  const VL tt = beach<T, VEC, KW>([](T a, T b) { return a - b; }, f, d);
+                                  bstore(L, t, r, tt);
+                                  bstore(L, w, r, beach<T, VEC, KW>([&](T a) { return ap * a; }, tt));
+                              });
 }
 
-template <class T, int KW, int PW>
+template <class T, int VEC, int KW, int PW>
 __global__ void kb_horner(SellView<T> A, const T* __restrict__ t, const T* __restrict__ win,
-                          T* __restrict__ wout, T ak, int k, int rev)
+                          T* __restrict__ wout, T ak, int k, int lg, int rev)
 {
-    bfor_rows<T, KW, PW>(A, win, k, true,
-                         [&](int r, int lane) { return row_vals<T, KW>(t, nullptr, r, -1, lane, k); },
-                         [&](int r, int lane, const T (&a)[KW], const RowVals<T, KW>& pv) {
-#pragma unroll
-        for (int j = 0; j < KW; ++j) {
-            int q = lane + 32 * j;
-            if (q < k) wout[size_t(r) * k + q] = fma(ak, pv.a[j], a[j]);
-        }
-    }, rev);
+    using LN = Lanes<T, VEC, KW>;
+    using VL = Vals<T, VEC, KW>;
+    bfor_rows<T, VEC, KW, PW>(A, win, k, lg, true, [&](int r, const LN& L) { return bload(L, t, r); },
+                              [&](int r, const LN& L, const VL& d, const VL& tv) {
+                                  bstore(L, wout, r, beach<T, VEC, KW>([&](T a, T b) { return fma(ak, a, b); }, tv, d));
+                              }, rev);
 }
 
-template <class T, int KW, int PW>
+template <class T, int VEC, int KW, int PW>
 __global__ void kb_horner_last(SellView<T> A, const T* __restrict__ t, const T* __restrict__ win,
                                const T* __restrict__ ec, const int* __restrict__ W,
-                               T* __restrict__ ef, T a0, int k, int rev)
+                               T* __restrict__ ef, T a0, int k, int lg, int rev)
 {
-    bfor_rows<T, KW, PW>(A, win, k, true,
-                         [&](int r, int lane) { return row_vals<T, KW>(t, ec, r, W[r], lane, k); },
-                         [&](int r, int lane, const T (&a)[KW], const RowVals<T, KW>& pv) {
-#pragma unroll
-        for (int j = 0; j < KW; ++j) {
-            int q = lane + 32 * j;
-            if (q < k) ef[size_t(r) * k + q] = pv.b[j] + fma(a0, pv.a[j], a[j]);
-        }
-    }, rev);
+    using LN = Lanes<T, VEC, KW>;
+    using VL = Vals<T, VEC, KW>;
+    using V2 = Vals2<T, VEC, KW>;
+    bfor_rows<T, VEC, KW, PW>(A, win, k, lg, true,
+                              [&](int r, const LN& L) { return V2{bload(L, t, r), bload(L, ec, W[r])}; },
+                              [&](int r, const LN& L, const VL& d, const V2& q) {
+                                  bstore(L, ef, r, beach<T, VEC, KW>([&](T e, T a, T b) { return e + fma(a0, a, b); },
+                                                                     q.b, q.a, d));
+                              }, rev);
 }
 
 // last Horner term of an in-place smoother: e += a_0 t + A win (C-point
 // smooth, second F-point smooth of FCF; with win = t and a_0 = 0 it applies
 // an assembled inverse)
-template <class T, int KW, int PW>
+template <class T, int VEC, int KW, int PW>
 __global__ void kb_horner_acc(SellView<T> A, const T* __restrict__ t, const T* __restrict__ win, T* e, T a0,
-                              int k, int rev)
+                              int k, int lg, int rev)
 {
-    bfor_rows<T, KW, PW>(A, win, k, true,
-                         [&](int r, int lane) { return row_vals<T, KW>(t, e, r, r, lane, k); },
-                         [&](int r, int lane, const T (&a)[KW], const RowVals<T, KW>& pv) {
-#pragma unroll
-        for (int j = 0; j < KW; ++j) {
-            int q = lane + 32 * j;
-            if (q < k) e[size_t(r) * k + q] = pv.b[j] + fma(a0, pv.a[j], a[j]);
-        }
-    }, rev);
+    using LN = Lanes<T, VEC, KW>;
+    using VL = Vals<T, VEC, KW>;
+    using V2 = Vals2<T, VEC, KW>;
+    bfor_rows<T, VEC, KW, PW>(A, win, k, lg, true,
+                              [&](int r, const LN& L) { return V2{bload(L, t, r), bload(L, (const T*)e, r)}; },
+                              [&](int r, const LN& L, const VL& d, const V2& q) {
+                                  bstore(L, e, r, beach<T, VEC, KW>([&](T ee, T a, T b) { return ee + fma(a0, a, b); },
+                                                                    q.b, q.a, d));
+                              }, rev);
 }
 
 // degree-0 in-place correction e += a_0 t, and a copy, over m values
@@ -264,58 +322,53 @@ __global__ void kb_smooth0(long long n, const T* __restrict__ t, const T* __rest
 }
 
 // Newton steps of the coarse polynomial (Sec. 2.3) for k right-hand sides
-template <class T, int KW, int PW>
+template <class T, int VEC, int KW, int PW>
 __global__ void kb_newton_real(SellView<T> A, const T* __restrict__ rin, T* __restrict__ rout,
-                               T* __restrict__ x, T inv, int first, int last, int k, int rev)
+                               T* __restrict__ x, T inv, int first, int last, int k, int lg, int rev)
 {
-    bfor_rows<T, KW, PW>(A, rin, k, !last,
-                         [&](int r, int lane) { return row_vals<T, KW>(rin, first ? nullptr : x, r, r, lane, k); },
-                         [&](int r, int lane, const T (&a)[KW], const RowVals<T, KW>& pv) {
-#pragma unroll
-        for (int j = 0; j < KW; ++j) {
-            int q = lane + 32 * j;
-            if (q < k) {
-                size_t o = size_t(r) * k + q;
-                x[o] = fma(pv.a[j], inv, pv.b[j]);
-                if (!last) rout[o] = pv.a[j] - a[j] * inv;
-            }
-        }
-    }, rev);
+    using LN = Lanes<T, VEC, KW>;
+    using VL = Vals<T, VEC, KW>;
+    using V2 = Vals2<T, VEC, KW>;
+    bfor_rows<T, VEC, KW, PW>(A, rin, k, lg, !last,
+                              [&](int r, const LN& L) {
+                                  return V2{bload(L, rin, r), bload(L, first ? (const T*)nullptr : (const T*)x, r)};
+                              },
+                              [&](int r, const LN& L, const VL& d, const V2& q) {
+                                  bstore(L, x, r, beach<T, VEC, KW>([&](T a, T b) { return fma(a, inv, b); }, q.a, q.b));
+                                  if (!last)
+                                      bstore(L, rout, r,
+                                             beach<T, VEC, KW>([&](T a, T b) { return a - b * inv; }, q.a, d));
+                              }, rev);
 }
 
-template <class T, int KW, int PW>
+template <class T, int VEC, int KW, int PW>
 __global__ void kb_newton_pair1(SellView<T> A, const T* __restrict__ rin, T* __restrict__ t,
-                                T* __restrict__ x, T two_a, T inv2, int first, int k, int rev)
+                                T* __restrict__ x, T two_a, T inv2, int first, int k, int lg, int rev)
 {
-    bfor_rows<T, KW, PW>(A, rin, k, true,
-                         [&](int r, int lane) { return row_vals<T, KW>(rin, first ? nullptr : x, r, r, lane, k); },
-                         [&](int r, int lane, const T (&a)[KW], const RowVals<T, KW>& pv) {
-#pragma unroll
-        for (int j = 0; j < KW; ++j) {
-            int q = lane + 32 * j;
-            if (q < k) {
-                size_t o = size_t(r) * k + q;
-                T tt = two_a * pv.a[j] - a[j];
-                t[o] = tt;
-                x[o] = fma(tt, inv2, pv.b[j]);
-            }
-        }
-    }, rev);
+    using LN = Lanes<T, VEC, KW>;
+    using VL = Vals<T, VEC, KW>;
+    using V2 = Vals2<T, VEC, KW>;
+    bfor_rows<T, VEC, KW, PW>(A, rin, k, lg, true,
+                              [&](int r, const LN& L) {
+                                  return V2{bload(L, rin, r), bload(L, first ? (const T*)nullptr : (const T*)x, r)};
+                              },
+                              [&](int r, const LN& L, const VL& d, const V2& q) {
+                                  const VL tt = beach<T, VEC, KW>([&](T a, T b) { return two_a * a - b; }, q.a, d);
+                                  bstore(L, t, r, tt);
+                                  bstore(L, x, r, beach<T, VEC, KW>([&](T a, T b) { return fma(a, inv2, b); }, tt, q.b));
+                              }, rev);
 }
 
-template <class T, int KW, int PW>
+template <class T, int VEC, int KW, int PW>
 __global__ void kb_newton_pair2(SellView<T> A, const T* __restrict__ rin, const T* __restrict__ t,
-                                T* __restrict__ rout, T inv2, int k, int rev)
+                                T* __restrict__ rout, T inv2, int k, int lg, int rev)
 {
-    bfor_rows<T, KW, PW>(A, t, k, true,
-                         [&](int r, int lane) { return row_vals<T, KW>(rin, nullptr, r, -1, lane, k); },
-                         [&](int r, int lane, const T (&a)[KW], const RowVals<T, KW>& pv) {
-#pragma unroll
-        for (int j = 0; j < KW; ++j) {
-            int q = lane + 32 * j;
-            if (q < k) rout[size_t(r) * k + q] = pv.a[j] - a[j] * inv2;
-        }
-    }, rev);
+    using LN = Lanes<T, VEC, KW>;
+    using VL = Vals<T, VEC, KW>;
+    bfor_rows<T, VEC, KW, PW>(A, t, k, lg, true, [&](int r, const LN& L) { return bload(L, rin, r); },
+                              [&](int r, const LN& L, const VL& d, const VL& ri) {
+                                  bstore(L, rout, r, beach<T, VEC, KW>([&](T a, T b) { return a - b * inv2; }, ri, d));
+                              }, rev);
 }
 
 __global__ void kb_d2f(long long m, const double* a, float* b)
@@ -510,19 +563,46 @@ __global__ void kb_sub(long long m, const double* b, const double* y, double* r)
     if (i < m) r[i] = b[i] - y[i];
 }
 
-#define WITH_KW(k, ...)                                                   \
-    do {                                                                  \
-        if ((k) <= 32) { constexpr int KW = 1; __VA_ARGS__; }             \
-        else if ((k) <= 64) { constexpr int KW = 2; __VA_ARGS__; }        \
-        else { constexpr int KW = 4; __VA_ARGS__; }                       \
-    } while (0)
+// Shape of a batch of k vectors of type T (Lanes): 16-byte packs where every
+// row of k values starts on a 16-byte boundary, the smallest power of two of
+// lanes that covers the packs, and KW steps of a whole warp beyond 32.
+struct BShape {
+    int vec, lg, kw;
+};
+template <class T>
+BShape bshape(int k)
+{
+    const int full = 16 / int(sizeof(T));
+    BShape s{k % full == 0 ? full : 1, 0, 1};
+    const int packs = k / s.vec;
+    while (s.lg < 5 && (1 << s.lg) < packs) ++s.lg;
+    s.kw = packs <= 32 ? 1 : (packs <= 64 ? 2 : 4);
+    return s;
+}
 
-// Runs the statement with KW (right-hand sides per lane) and PW (warps per
-// row: 1 for operators with short rows, 4 for long rows) of operator S.
-#define WITH_KWPW(k, S, ...)                                              \
-    do {                                                                  \
-        if ((S).k == 1) { constexpr int PW = 1; WITH_KW(k, __VA_ARGS__); } \
-        else { constexpr int PW = 4; WITH_KW(k, __VA_ARGS__); }           \
+// Runs the statement with VEC, KW and lg of a batch of k vectors of type T,
+// and PW (warps per row: 1 for operators with short rows, 4 for long rows)
+// of operator S.  (16-byte packs: at most 128 / 4 FP32 or 128 / 2 FP64
+// lanes, so KW = 1, or 2 in FP64.)
+#define WITH_SHAPE(T, bs, ...)                                                       \
+    do {                                                                             \
+        if ((bs).vec == 1) {                                                         \
+            constexpr int VEC = 1;                                                   \
+            if ((bs).kw == 1) { constexpr int KW = 1; __VA_ARGS__; }                 \
+            else if ((bs).kw == 2) { constexpr int KW = 2; __VA_ARGS__; }            \
+            else { constexpr int KW = 4; __VA_ARGS__; }                              \
+        } else {                                                                     \
+            constexpr int VEC = 16 / int(sizeof(T));                                 \
+            if ((bs).kw == 1) { constexpr int KW = 1; __VA_ARGS__; }                 \
+            else { constexpr int KW = sizeof(T) == 8 ? 2 : 1; __VA_ARGS__; }         \
+        }                                                                            \
+    } while (0)
+#define WITH_BATCH(T, k, S, ...)                                                     \
+    do {                                                                             \
+        const BShape bs_ = bshape<T>(k);                                             \
+        const int lg = bs_.lg;                                                       \
+        if ((S).k == 1) { constexpr int PW = 1; WITH_SHAPE(T, bs_, __VA_ARGS__); }   \
+        else { constexpr int PW = 4; WITH_SHAPE(T, bs_, __VA_ARGS__); }              \
     } while (0)
 
 }  // namespace
@@ -583,13 +663,13 @@ void bf_smooth(SolveData& S, int l, int k, const T* v, T* e, const BWork<T>& wk,
     const long long fB = (long long)nf * VB * kk;
     S.cur_level = l;
     LAUNCH_F(S, PK_FRESID, mat_bytes32(o.M) + (long long)lv.n_c * VB * kk + 3 * fB, (2 * o.M.nnz + 2LL * nf) * kk,
-           WITH_KWPW(k, o.M, kb_fresid<T, KW, PW><<<grid_rows(nf, PW), BT, 0, st>>>(view(o.M), rf, ec, wk.t, wk.wa,
-                                                                    T(lv.alpha[p]), k)));
+           WITH_BATCH(T, k, o.M, kb_fresid<T, VEC, KW, PW><<<grid_rows(nf, PW, lg), BT, 0, st>>>(view(o.M), rf, ec, wk.t, wk.wa,
+                                                                    T(lv.alpha[p]), k, lg)));
     if (o.Ainv.n_rows) {
         // assembled smoother: e_f = W e_c + Ahat^-1 t (last Horner kernel, a0 = 0)
         LAUNCH_F(S, PK_HORNER, mat_bytes32(o.Ainv) + 4 * fB + 4LL * nf, (2 * o.Ainv.nnz + 3LL * nf) * kk,
-                 WITH_KWPW(k, o.Ainv, kb_horner_last<T, KW, PW><<<grid_rows(nf, PW), BT, 0, st>>>(view(o.Ainv), wk.t, wk.t, ec,
-                                                                               lv.W.p, ef, T(0), k, 0)));
+                 WITH_BATCH(T, k, o.Ainv, kb_horner_last<T, VEC, KW, PW><<<grid_rows(nf, PW, lg), BT, 0, st>>>(view(o.Ainv), wk.t, wk.t, ec,
+                                                                               lv.W.p, ef, T(0), k, lg, 0)));
         return;
     }
     if (p == 0) {
@@ -603,13 +683,13 @@ void bf_smooth(SolveData& S, int l, int k, const T* v, T* e, const BWork<T>& wk,
     T* wout = wk.wb;
     for (int kq = p - 1; kq >= 1; --kq) {
         LAUNCH_F(S, PK_HORNER, hB, (2 * o.Aff.nnz + 2LL * nf) * kk,
-               WITH_KWPW(k, o.Aff, kb_horner<T, KW, PW><<<grid_rows(nf, PW), BT, 0, st>>>(view(o.Aff), wk.t, win, wout,
-                                                                        T(lv.alpha[kq]), k, serpentine(p - 1 - kq))));
+               WITH_BATCH(T, k, o.Aff, kb_horner<T, VEC, KW, PW><<<grid_rows(nf, PW, lg), BT, 0, st>>>(view(o.Aff), wk.t, win, wout,
+                                                                        T(lv.alpha[kq]), k, lg, serpentine(p - 1 - kq))));
         std::swap(win, wout);
     }
     LAUNCH_F(S, PK_HORNER, hB + fB + 4LL * nf, (2 * o.Aff.nnz + 3LL * nf) * kk,
-           WITH_KWPW(k, o.Aff, kb_horner_last<T, KW, PW><<<grid_rows(nf, PW), BT, 0, st>>>(view(o.Aff), wk.t, win, ec,
-                                                                         lv.W.p, ef, T(lv.alpha[0]), k, serpentine(p - 1))));
+           WITH_BATCH(T, k, o.Aff, kb_horner_last<T, VEC, KW, PW><<<grid_rows(nf, PW, lg), BT, 0, st>>>(view(o.Aff), wk.t, win, ec,
+                                                                         lv.W.p, ef, T(lv.alpha[0]), k, lg, serpentine(p - 1))));
 }
 
 // e += q(A) t by Horner for k right-hand sides, w = a_p t already in wk.wa
@@ -630,13 +710,13 @@ void bhorner_into(SolveData& S, const Sell<T>& A, const std::vector<double>& al,
     T* wout = wk.wb;
     for (int kq = p - 1; kq >= 1; --kq) {
         LAUNCH_F(S, PK_HORNER, hB, (2 * A.nnz + 2LL * n) * kk,
-                 WITH_KWPW(k, A, kb_horner<T, KW, PW><<<grid_rows(n, PW), BT, 0, st>>>(view(A), wk.t, win, wout,
-                                                                                      T(al[kq]), k, serpentine(p - 1 - kq))));
+                 WITH_BATCH(T, k, A, kb_horner<T, VEC, KW, PW><<<grid_rows(n, PW, lg), BT, 0, st>>>(view(A), wk.t, win, wout,
+                                                                                      T(al[kq]), k, lg, serpentine(p - 1 - kq))));
         std::swap(win, wout);
     }
     LAUNCH_F(S, PK_HORNER, hB + fB, (2 * A.nnz + 3LL * n) * kk,
-             WITH_KWPW(k, A, kb_horner_acc<T, KW, PW><<<grid_rows(n, PW), BT, 0, st>>>(view(A), wk.t, win, e,
-                                                                                      T(al[0]), k, serpentine(p - 1))));
+             WITH_BATCH(T, k, A, kb_horner_acc<T, VEC, KW, PW><<<grid_rows(n, PW, lg), BT, 0, st>>>(view(A), wk.t, win, e,
+                                                                                      T(al[0]), k, lg, serpentine(p - 1))));
 }
 
 // C-point smooth of level l for k right-hand sides (Sec. 2):
@@ -657,12 +737,12 @@ void bc_smooth(SolveData& S, int l, int k, const T* v, T* e, const BWork<T>& wk,
     const long long cB = (long long)nc * VB * kk;
     LAUNCH_F(S, PK_FRESID, mat_bytes32(o.Mc) + (long long)(lv.n_f + nc) * VB * kk + 3 * cB,
              (2 * o.Mc.nnz + 2LL * nc) * kk,
-             WITH_KWPW(k, o.Mc, kb_fresid<T, KW, PW><<<grid_rows(nc, PW), BT, 0, st>>>(view(o.Mc), rc, el, wk.t, wk.wa,
-                                                                                   T(lv.alpha_c[p]), k)));
+             WITH_BATCH(T, k, o.Mc, kb_fresid<T, VEC, KW, PW><<<grid_rows(nc, PW, lg), BT, 0, st>>>(view(o.Mc), rc, el, wk.t, wk.wa,
+                                                                                   T(lv.alpha_c[p]), k, lg)));
     if (o.Ainvc.n_rows) {
         LAUNCH_F(S, PK_HORNER, mat_bytes32(o.Ainvc) + 4 * cB, (2 * o.Ainvc.nnz + 2LL * nc) * kk,
-                 WITH_KWPW(k, o.Ainvc, kb_horner_acc<T, KW, PW><<<grid_rows(nc, PW), BT, 0, st>>>(
-                                           view(o.Ainvc), wk.t, wk.t, ec, T(0), k, 0)));
+                 WITH_BATCH(T, k, o.Ainvc, kb_horner_acc<T, VEC, KW, PW><<<grid_rows(nc, PW, lg), BT, 0, st>>>(
+                                           view(o.Ainvc), wk.t, wk.t, ec, T(0), k, lg, 0)));
         return;
     }
     bhorner_into<T>(S, o.Acc, lv.alpha_c, wk, ec, nc, k, st);
@@ -684,12 +764,12 @@ void bf_smooth_again(SolveData& S, int l, int k, const T* v, T* e, const BWork<T
     const long long fB = (long long)nf * VB * kk;
     LAUNCH_F(S, PK_FRESID, mat_bytes32(o.Mf) + (long long)(nf + lv.n_c) * VB * kk + 3 * fB,
              (2 * o.Mf.nnz + 2LL * nf) * kk,
-             WITH_KWPW(k, o.Mf, kb_fresid<T, KW, PW><<<grid_rows(nf, PW), BT, 0, st>>>(view(o.Mf), rf, el, wk.t, wk.wa,
-                                                                                   T(lv.alpha[p]), k)));
+             WITH_BATCH(T, k, o.Mf, kb_fresid<T, VEC, KW, PW><<<grid_rows(nf, PW, lg), BT, 0, st>>>(view(o.Mf), rf, el, wk.t, wk.wa,
+                                                                                   T(lv.alpha[p]), k, lg)));
     if (o.Ainv.n_rows) {
         LAUNCH_F(S, PK_HORNER, mat_bytes32(o.Ainv) + 4 * fB, (2 * o.Ainv.nnz + 2LL * nf) * kk,
-                 WITH_KWPW(k, o.Ainv, kb_horner_acc<T, KW, PW><<<grid_rows(nf, PW), BT, 0, st>>>(
-                                          view(o.Ainv), wk.t, wk.t, el, T(0), k, 0)));
+                 WITH_BATCH(T, k, o.Ainv, kb_horner_acc<T, VEC, KW, PW><<<grid_rows(nf, PW, lg), BT, 0, st>>>(
+                                          view(o.Ainv), wk.t, wk.t, el, T(0), k, lg, 0)));
         return;
     }
     bhorner_into<T>(S, o.Aff, lv.alpha, wk, el, nf, k, st);
@@ -715,15 +795,15 @@ void bvcycle(SolveData& S, int k, const T* v, T* e, const BWork<T>& wk, cudaStre
         if (lv.n_c && Zb.val.n)
             LAUNCH_F(S, PK_RESTRICT, mat_bytes32(Zb) + (2LL * lv.n_c + lv.n_f + lv.n_c) * VB * kk,
                      (2 * Zb.nnz + lv.n_c) * kk,
-                     WITH_KWPW(k, Zb, kb_restrict<T, KW, PW, bf16s><<<grid_rows(lv.n_c, PW), BT, 0, st>>>(
+                     WITH_BATCH(T, k, Zb, kb_restrict<T, VEC, KW, PW, bf16s><<<grid_rows(lv.n_c, PW, lg), BT, 0, st>>>(
                                     view(Zb), src + size_t(lv.off) * k, src + size_t(lv.off + lv.n_f) * k,
-                                    wk.rwork + size_t(lv.off + lv.n_f) * k, k)));
+                                    wk.rwork + size_t(lv.off + lv.n_f) * k, k, lg)));
         else if (lv.n_c)
             LAUNCH_F(S, PK_RESTRICT, mat_bytes32(Z) + (2LL * lv.n_c + lv.n_f + lv.n_c) * VB * kk,
                      (2 * Z.nnz + lv.n_c) * kk,
-                   WITH_KWPW(k, Z, kb_restrict<T, KW, PW><<<grid_rows(lv.n_c, PW), BT, 0, st>>>(
+                   WITH_BATCH(T, k, Z, kb_restrict<T, VEC, KW, PW><<<grid_rows(lv.n_c, PW, lg), BT, 0, st>>>(
                                   view(Z), src + size_t(lv.off) * k, src + size_t(lv.off + lv.n_f) * k,
-                                  wk.rwork + size_t(lv.off + lv.n_f) * k, k)));
+                                  wk.rwork + size_t(lv.off + lv.n_f) * k, k, lg)));
     }
     {
         const T* rc = (L == 0 ? v : wk.rwork) + size_t(S.off_c) * k;
@@ -745,18 +825,18 @@ void bvcycle(SolveData& S, int k, const T* v, T* e, const BWork<T>& wk, cudaStre
             if (q.im == 0.0) {
                 LAUNCH_F(S, PK_NEWTON, (last ? 0 : mB + 2 * nB) + (i == 0 ? 2 : 3) * nB,
                          (last ? 2LL * nco : 2 * A.nnz + 4LL * nco) * kk,
-                       WITH_KWPW(k, A, kb_newton_real<T, KW, PW><<<grid_rows(nco, PW), BT, 0, st>>>(
-                                      Av, rin, rout, x, T(1.0 / q.re), i == 0, last, k, serpentine(nsp))));
+                       WITH_BATCH(T, k, A, kb_newton_real<T, VEC, KW, PW><<<grid_rows(nco, PW, lg), BT, 0, st>>>(
+                                      Av, rin, rout, x, T(1.0 / q.re), i == 0, last, k, lg, serpentine(nsp))));
                 nsp += 1;
             } else {
                 double mod2 = q.re * q.re + q.im * q.im;
                 LAUNCH_F(S, PK_NEWTON, mB + (i == 0 ? 3 : 4) * nB, (2 * A.nnz + 4LL * nco) * kk,
-                       WITH_KWPW(k, A, kb_newton_pair1<T, KW, PW><<<grid_rows(nco, PW), BT, 0, st>>>(
-                                      Av, rin, wk.ct, x, T(2.0 * q.re), T(1.0 / mod2), i == 0, k, serpentine(nsp))));
+                       WITH_BATCH(T, k, A, kb_newton_pair1<T, VEC, KW, PW><<<grid_rows(nco, PW, lg), BT, 0, st>>>(
+                                      Av, rin, wk.ct, x, T(2.0 * q.re), T(1.0 / mod2), i == 0, k, lg, serpentine(nsp))));
                 if (!last)
                     LAUNCH_F(S, PK_NEWTON, mB + 3 * nB, (2 * A.nnz + 2LL * nco) * kk,
-                           WITH_KWPW(k, A, kb_newton_pair2<T, KW, PW><<<grid_rows(nco, PW), BT, 0, st>>>(
-                                          Av, rin, wk.ct, rout, T(1.0 / mod2), k, serpentine(nsp + 1))));
+                           WITH_BATCH(T, k, A, kb_newton_pair2<T, VEC, KW, PW><<<grid_rows(nco, PW, lg), BT, 0, st>>>(
+                                          Av, rin, wk.ct, rout, T(1.0 / mod2), k, lg, serpentine(nsp + 1))));
                 nsp += 2;
             }
             if (!last) { rin = rout; nb ^= 1; }
@@ -898,7 +978,7 @@ void solve_batched(Hierarchy& H, int k, const double* b, double* x, double rtol,
     for (int q = 0; q < k; ++q) tol[q] = std::max(rtol * bn[q], atol);
     auto residual = [&]() {
         LAUNCH_F(S, PK_TOPSPMV, topB, 2 * S.Atop.nnz * k,
-               WITH_KWPW(k, S.Atop, kb_spmv<double, KW, PW><<<grid_rows(n, PW), BT, 0, st>>>(A, B.xp.p, B.w.p, k)));
+               WITH_BATCH(double, k, S.Atop, kb_spmv<double, VEC, KW, PW><<<grid_rows(n, PW, lg), BT, 0, st>>>(A, B.xp.p, B.w.p, k, lg)));
         LAUNCH_F(S, PK_KRYLOV, 24 * nk, nk, kb_sub<<<g, BT, 0, st>>>(nk, B.bp.p, B.w.p, B.r.p));
         bnorms(S, B, B.r.p, rn, st);
     };
@@ -944,7 +1024,7 @@ void solve_batched(Hierarchy& H, int k, const double* b, double* x, double rtol,
             double* zj = B.Zs.p + size_t(j) * nk;
             bprecond(H, B, vj, zj, st);
             LAUNCH_F(S, PK_TOPSPMV, topB, 2 * S.Atop.nnz * k,
-                   WITH_KWPW(k, S.Atop, kb_spmv<double, KW, PW><<<grid_rows(n, PW), BT, 0, st>>>(A, zj, B.w.p, k)));
+                   WITH_BATCH(double, k, S.Atop, kb_spmv<double, VEC, KW, PW><<<grid_rows(n, PW, lg), BT, 0, st>>>(A, zj, B.w.p, k, lg)));
             // CGS with a second pass only if the first cancelled, for some
             // active right-hand side, more than reorth_ratio() allows
             double* h1 = B.hdev.p;
