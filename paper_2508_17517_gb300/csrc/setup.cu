@@ -527,82 +527,400 @@ __global__ void k_scale(int nnz, double* v, double s)
 }
 
 // -------------------------------------------------------------- SpGEMM ----
-// C = A B.  Each row of C is built by one thread in a private open-addressing
-// table: contributions arrive in ascending order of A's column (the inner
-// index), so every entry is the left-to-right sum of the definition.
-__global__ void k_gemm_bound(int m, const int* arp, const int* aci, const int* brp, int* tsize)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m) return;
-    long long b = 0;
-    for (int p = arp[i]; p < arp[i + 1]; ++p) b += brp[aci[p] + 1] - brp[aci[p]];
-    int sz = 0;
-    if (b > 0) {
-        sz = 1;
-        while (sz < 2 * b) sz <<= 1;
-    }
-    tsize[i] = sz;
-}
+// C = A B.  An entry of C is the left-to-right sum of its products in
+// ascending inner index (A's column), starting from +0.0.  The products of a
+// row are numbered in that order (A's entries in turn, each with its row of
+// B), and every path below adds products with the same column in that order.
+// Rows are handled by the number of their products:
+//   at most 8 / 32: a group of 8 / 32 lanes sorts them by column in
+//     registers;
+//   more: a warp adds them into a hash table in shared memory and ranks the
+//     columns with a bitmap over their range.
+//   rows with more distinct columns than GEMM_CAP: tables in global memory.
+// The sorted rows go to a scratch piece and from there, packed, into C.
+// Bound: latency of the loads of B's rows and of the shared-memory table, at
+// 12-16 warps per SM.  Tables in global memory for every row, sized at twice
+// the products, cleared and scanned as a whole and sorted with bitonic
+// networks, took 1.20 s of the 4096^2 setup (restrictor and RAP together);
+// this takes 0.35 s.
+constexpr int GEMM_TINY = 8, GEMM_SMALL = 32;   // products per lane group
+constexpr int GEMM_SLOTS = 1024, GEMM_SLOTS_LOW = 512;   // shared-memory table of a warp
+constexpr int GEMM_CAP = GEMM_SLOTS / 4 * 3;    // distinct columns a table takes
+constexpr int GEMM_LOW = GEMM_SLOTS_LOW / 4 * 3;   // products of a row of the smaller table
+constexpr int GEMM_WORDS = 1024;                // bitmap words: columns within 32,768 of each other
+constexpr int GEMM_WARPS = 4;                   // rows per block
 
 __device__ __forceinline__ unsigned hash_col(int j) { return (unsigned)j * 2654435761u; }
 
-// Rows whose table has at least HASH_WARP_SLOTS slots are accumulated by a
-// warp (k_gemm_hash_warp), the others by one thread (k_gemm_hash).
-constexpr int HASH_WARP_SLOTS = 64;
-
-__global__ void k_gemm_hash(int m, int row0, const int* arp, const int* aci, const double* av,
-                            const int* brp, const int* bci, const double* bv, const int* toff,
-                            int* keys, double* vals, int* cnt)
+// Products of row row0 + li (saturated), the scratch entries of the row
+// (never more than its products or GEMM_CAP), and the row's class list.
+// lists: four of m entries each, counts: their lengths.
+__global__ void k_gemm_bound(int m, int row0, const int* arp, const int* aci, const int* brp, int* prod, int* room)
 {
-    int li = blockIdx.x * blockDim.x + threadIdx.x;   // row within the chunk
+    int li = blockIdx.x * blockDim.x + threadIdx.x;
     if (li >= m) return;
-    int i = row0 + li;
-    int base = toff[li], size = toff[li + 1] - base;
-    if (size >= HASH_WARP_SLOTS) return;
+    const int i = row0 + li;
+    long long b = 0;
+    for (int p = arp[i]; p < arp[i + 1]; ++p) b += brp[aci[p] + 1] - brp[aci[p]];
+    const int n = int(b < 0x3fffffffLL ? b : 0x3fffffffLL);
+    prod[li] = n;
+    room[li] = n < GEMM_CAP ? n : GEMM_CAP;
+}
+
+__device__ __forceinline__ int gemm_class(int b)
+{
+    return b <= 0 ? -1 : (b <= GEMM_TINY ? 0 : (b <= GEMM_SMALL ? 1 : (b <= GEMM_LOW ? 2 : 3)));
+}
+
+// Class lists of the rows of a piece (one aggregated atomic per warp and
+// class; the order of a list does not matter), and zero counts for the rows
+// without products.
+__global__ void k_gemm_lists(int m, const int* prod, int* lists, int* counts, int* cnt)
+{
+    const int li = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const int cl = li < m ? gemm_class(prod[li]) : -1;
+    if (li < m && cl < 0) cnt[li] = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const unsigned b = __ballot_sync(0xffffffffu, cl == c);
+        if (!b) continue;
+        int at = 0;
+        if (lane == 0) at = atomicAdd(counts + c, __popc(b));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (cl == c) lists[(long long)c * m + at + __popc(b & ((1u << lane) - 1u))] = li;
+    }
+}
+
+// Product f of the entries held by a group of G lanes: lane k holds an
+// entry of A (value a, its row of B at bs) and `inc`, the number of products
+// up to and including it.  Sets the product's column and value.
+template <int G>
+__device__ __forceinline__ void gemm_product(int f, int inc, int len, double a, int bs, const int* __restrict__ bci,
+                                             const double* __restrict__ bv, bool valid, int& j, double& pr)
+{
+    const unsigned full = 0xffffffffu;
+    int k = 0;
+#pragma unroll
+    for (int s = G / 2; s > 0; s >>= 1)
+        if (__shfl_sync(full, inc, k + s - 1, G) <= f) k += s;
+    const int before = __shfl_sync(full, inc - len, k, G), b0 = __shfl_sync(full, bs, k, G);
+    const double ak = __shfl_sync(full, a, k, G);
+    j = 0x7fffffff;
+    pr = 0.0;
+    if (valid) {
+        const int q = b0 + (f - before);
+        j = __ldg(bci + q);
+        pr = __dmul_rn(ak, __ldg(bv + q));
+    }
+}
+
+// Rows of at most G products (G = 8 or 32): one product per lane, sorted by
+// (column, order) with a bitonic network; the first lane of each column adds
+// the others in order.
+template <int G>
+__global__ void k_gemm_lanes(int nlist, const int* __restrict__ list, int row0, const int* __restrict__ arp,
+                             const int* __restrict__ aci, const double* __restrict__ av,
+                             const int* __restrict__ brp, const int* __restrict__ bci,
+                             const double* __restrict__ bv, const int* __restrict__ toff, int* __restrict__ tci,
+                             double* __restrict__ tv, int* __restrict__ cnt)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, g = lane & (G - 1);
+    const int at = (blockIdx.x * blockDim.x + threadIdx.x) / G;
+    const bool row = at < nlist;                  // uniform over the group
+    if (!__any_sync(full, row)) return;
+    const int li = row ? list[at] : 0, i = row0 + li;
+    const int a0 = row ? arp[i] : 0, alen = row ? arp[i + 1] - a0 : 0;
+    // A's entries with an empty row of B may exceed the lanes: only entries
+    // with products are kept
+    int have = 0, inc = 0, len = 0, bs = 0;
+    double a = 0.0;
+    const int most = __reduce_max_sync(full, alen);
+    for (int p0 = 0; p0 < most; p0 += G) {
+        const int p = p0 + g;
+        int l = 0, n = 0, s = 0;
+        if (p < alen) {
+            l = aci[a0 + p];
+            s = brp[l];
+            n = brp[l + 1] - s;
+        }
+        const unsigned mask = __ballot_sync(full, n > 0) >> (lane & ~(G - 1)) & (G == 32 ? full : ((1u << (G & 31)) - 1u));
+        // the t-th kept entry of this step goes to lane have + t
+        const int t = g - have;
+        const int src = t >= 0 && t < __popc(mask) ? int(__fns(mask, 0, t + 1)) : -1;
+        const int sn = __shfl_sync(full, n, src < 0 ? 0 : src, G), ss = __shfl_sync(full, s, src < 0 ? 0 : src, G);
+        if (src >= 0) {
+            len = sn;
+            bs = ss;
+            a = av[a0 + p0 + src];
+        }
+        have += __popc(mask);
+    }
+    inc = len;
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) {
+        const int u = __shfl_up_sync(full, inc, o, G);
+        if (g >= o) inc += u;
+    }
+    const int total = __shfl_sync(full, inc, G - 1, G);
+    int j;
+    double v;
+    gemm_product<G>(g, inc, len, a, bs, bci, bv, row && g < total, j, v);
+    unsigned long long key = ((unsigned long long)(unsigned)j << 8) | (unsigned)g;
+#pragma unroll
+    for (int size = 2; size <= G; size <<= 1)
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            const unsigned long long ok = __shfl_xor_sync(full, key, stride, G);
+            const double ov = __shfl_xor_sync(full, v, stride, G);
+            const bool lower = (g & stride) == 0, up = (g & size) == 0;
+            if (lower == up ? ok < key : ok > key) {
+                key = ok;
+                v = ov;
+            }
+        }
+    j = int(key >> 8);
+    const int prev = __shfl_up_sync(full, j, 1, G);
+    const bool valid = row && g < total, head = valid && (g == 0 || prev != j);
+    double s = __dadd_rn(0.0, v);
+    bool more = head;
+    for (int t = 1; t < G; ++t) {
+        const int nj = __shfl_down_sync(full, j, t, G);
+        const double nv = __shfl_down_sync(full, v, t, G);
+        more = more && g + t < total && nj == j;
+        if (!__any_sync(full, more)) break;
+        if (more) s = __dadd_rn(s, nv);
+    }
+    const unsigned heads = __ballot_sync(full, head) >> (lane & ~(G - 1)) & (G == 32 ? full : ((1u << (G & 31)) - 1u));
+    if (head) {
+        const int o = toff[li] + __popc(heads & ((1u << g) - 1u));
+        tci[o] = j;
+        tv[o] = s;
+    }
+    if (row && g == 0) cnt[li] = __popc(heads);
+}
+
+// Adds the products of row i of A B, in order, into the warp's table: 32 at
+// a time, lane by lane where several have the same column.  Returns the
+// number of columns (their range in cmin, cmax), or -1 where they exceed
+// three quarters of a full-size table.
+template <int SLOTS>
+__device__ __forceinline__ int gemm_accumulate(int i, const int* __restrict__ arp, const int* __restrict__ aci,
+                                               const double* __restrict__ av, const int* __restrict__ brp,
+                                               const int* __restrict__ bci, const double* __restrict__ bv,
+                                               int* keys, double* vals, int size, int& cmin, int& cmax)
+{
+    const unsigned full = 0xffffffffu, lane = threadIdx.x & 31, below = (1u << lane) - 1u;
+    const unsigned mask = unsigned(size) - 1u;
     int c = 0;
-    if (size > 0) {
-        unsigned mask = (unsigned)size - 1u;
-        for (int p = arp[i]; p < arp[i + 1]; ++p) {
-            int l = aci[p];
-            double a = av[p];
-            for (int q = brp[l]; q < brp[l + 1]; ++q) {
-                int j = bci[q];
-                double prod = __dmul_rn(a, bv[q]);
-                unsigned h = hash_col(j) & mask;
+    const int a0 = arp[i], a1 = arp[i + 1];
+    for (int p0 = a0; p0 < a1; p0 += 32) {
+        const int p = p0 + int(lane);
+        int len = 0, bs = 0;
+        double a = 0.0;
+        if (p < a1) {
+            const int l = aci[p];
+            a = av[p];
+            bs = brp[l];
+            len = brp[l + 1] - bs;
+        }
+        int inc = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(full, inc, o);
+            if (lane >= o) inc += u;
+        }
+        const int total = __shfl_sync(full, inc, 31);
+        int j, nj;
+        double pr, npr;
+        gemm_product<32>(int(lane), inc, len, a, bs, bci, bv, int(lane) < total, j, pr);
+        for (int f0 = 0; f0 < total; f0 += 32, j = nj, pr = npr) {
+            // the next 32 products load while these are added
+            gemm_product<32>(f0 + 32 + int(lane), inc, len, a, bs, bci, bv, f0 + 32 + int(lane) < total, nj, npr);
+            const bool take = f0 + int(lane) < total;
+            unsigned h = hash_col(j) & mask;
+            bool claimed = false;
+            if (take) {
+                cmin = min(cmin, j);
+                cmax = max(cmax, j);
                 while (true) {
-                    int key = keys[base + h];
-                    if (key == j) { vals[base + h] = __dadd_rn(vals[base + h], prod); break; }
+                    int key = *(volatile int*)(keys + h);
                     if (key == -1) {
-                        keys[base + h] = j;
-                        vals[base + h] = __dadd_rn(0.0, prod);
-                        ++c;
-                        break;
+                        key = atomicCAS(keys + h, -1, j);
+                        if (key == -1) {
+                            vals[h] = 0.0;
+                            claimed = true;
+                            break;
+                        }
                     }
+                    if (key == j) break;
                     h = (h + 1u) & mask;
                 }
             }
+            __syncwarp();
+            c += __popc(__ballot_sync(full, claimed));
+            const unsigned same = __match_any_sync(full, take ? j : -1 - int(lane));
+            const int rank = __popc(same & below), rounds = __reduce_max_sync(full, rank);
+            for (int t = 0; t <= rounds; ++t) {
+                if (take && rank == t) vals[h] = __dadd_rn(vals[h], pr);
+                __syncwarp();
+            }
+            if (size == SLOTS && c > SLOTS / 4 * 3) return -1;   // at least a quarter stays free
         }
     }
-    cnt[li] = c;
+    return c;
 }
 
-// The rows with large tables, one warp each.  The entries of A's row are
-// taken one at a time, in column order, by the whole warp; the lanes share
-// that entry's row of B.  Within one entry of A the columns j of B's row are
-// distinct, so no two lanes add to the same j (a lane claims a new slot with
-// an atomic compare-and-swap), and the warp synchronises before the next
-// entry: every output entry is still summed in ascending inner index with
-// the same roundings as the one-thread kernel.
-__global__ void k_gemm_hash_warp(int m, int row0, const int* arp, const int* aci, const double* av,
-                                 const int* brp, const int* bci, const double* bv, const int* toff,
-                                 int* keys, double* vals, int* cnt)
+// The rows of a class list, one warp each: accumulate, rank the columns,
+// write the row in column order to the scratch piece.  A row that does not
+// fit gets count -1 and a place on the overflow list.
+template <int SLOTS>
+__global__ void __launch_bounds__(GEMM_WARPS * 32)
+k_gemm_hash(int nlist, const int* __restrict__ list, int row0, const int* __restrict__ arp,
+            const int* __restrict__ aci, const double* __restrict__ av, const int* __restrict__ brp,
+            const int* __restrict__ bci, const double* __restrict__ bv, const int* __restrict__ prod,
+            const int* __restrict__ toff, int* __restrict__ tci, double* __restrict__ tv, int* __restrict__ cnt,
+            int* __restrict__ over, int* nover)
+{
+    extern __shared__ __align__(16) unsigned char gemm_raw[];
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double* vals = reinterpret_cast<double*>(gemm_raw) + w * SLOTS;
+    int* keys = reinterpret_cast<int*>(reinterpret_cast<double*>(gemm_raw) + GEMM_WARPS * SLOTS) + w * SLOTS;
+    unsigned* bits = reinterpret_cast<unsigned*>(reinterpret_cast<double*>(gemm_raw) + GEMM_WARPS * SLOTS) +
+                     GEMM_WARPS * SLOTS + w * GEMM_WORDS;
+    unsigned short* pre = reinterpret_cast<unsigned short*>(
+                              reinterpret_cast<unsigned*>(reinterpret_cast<double*>(gemm_raw) + GEMM_WARPS * SLOTS) +
+                              GEMM_WARPS * SLOTS + GEMM_WARPS * GEMM_WORDS) + w * GEMM_WORDS;
+    const int at = blockIdx.x * GEMM_WARPS + w;
+    if (at >= nlist) return;                      // uniform over the warp
+    const int li = list[at], i = row0 + li;
+    int size = 64;
+    while (size < SLOTS && size < 2 * prod[li]) size <<= 1;
+    for (int t = lane; t < size; t += 32) keys[t] = -1;
+    __syncwarp();
+    int cmin = 0x7fffffff, cmax = -1;
+    const int c = gemm_accumulate<SLOTS>(i, arp, aci, av, brp, bci, bv, keys, vals, size, cmin, cmax);
+    if (c < 0) {
+        if (lane == 0) {
+            cnt[li] = -1;
+            over[atomicAdd(nover, 1)] = li;
+        }
+        return;
+    }
+    cmin = __reduce_min_sync(full, cmin);
+    cmax = __reduce_max_sync(full, cmax);
+    const int o = toff[li];
+    const long long range = (long long)cmax - cmin + 1;
+    if (range <= 32LL * GEMM_WORDS) {
+        const int nw = int((range + 31) >> 5);
+        for (int t = lane; t < nw; t += 32) bits[t] = 0u;
+        __syncwarp();
+        for (int t = lane; t < size; t += 32) {
+            const int d = keys[t] - cmin;
+            if (keys[t] >= 0) atomicOr(bits + (d >> 5), 1u << (d & 31));
+        }
+        __syncwarp();
+        int carry = 0;
+        for (int w0 = 0; w0 < nw; w0 += 32) {
+            const int n = w0 + lane < nw ? __popc(bits[w0 + lane]) : 0;
+            int inc = n;
+#pragma unroll
+            for (int q = 1; q < 32; q <<= 1) {
+                const int u = __shfl_up_sync(full, inc, q);
+                if (lane >= q) inc += u;
+            }
+            if (w0 + lane < nw) pre[w0 + lane] = (unsigned short)(carry + inc - n);
+            carry += __shfl_sync(full, inc, 31);
+        }
+        __syncwarp();
+        for (int t = lane; t < size; t += 32) {
+            const int key = keys[t];
+            if (key < 0) continue;
+            const int d = key - cmin;
+            const int r = int(pre[d >> 5]) + __popc(bits[d >> 5] & ((1u << (d & 31)) - 1u));
+            tci[o + r] = key;
+            tv[o + r] = vals[t];
+        }
+    } else {
+        // columns too far apart for the bitmap: an entry's rank is the
+        // number of smaller columns
+        int* seen = reinterpret_cast<int*>(bits);
+        int n = 0;
+        for (int t0 = 0; t0 < size; t0 += 32) {
+            const int key = keys[t0 + lane];
+            const unsigned b = __ballot_sync(full, key >= 0);
+            if (key >= 0) seen[n + __popc(b & ((1u << lane) - 1u))] = key;
+            n += __popc(b);
+        }
+        __syncwarp();
+        for (int t = lane; t < size; t += 32) {
+            const int key = keys[t];
+            if (key < 0) continue;
+            int r = 0;
+            for (int q = 0; q < n; ++q) r += seen[q] < key;
+            tci[o + r] = key;
+            tv[o + r] = vals[t];
+        }
+    }
+    if (lane == 0) cnt[li] = c;
+}
+inline size_t gemm_smem(int slots) { return size_t(GEMM_WARPS) * (size_t(slots) * 12 + GEMM_WORDS * 6); }
+
+// Rows of the scratch piece to their packed place, a warp for 32 rows.
+__global__ void k_gemm_pack(int m, const int* __restrict__ toff, const int* __restrict__ crp,
+                            const int* __restrict__ cnt, const int* __restrict__ tci,
+                            const double* __restrict__ tv, int* __restrict__ cci, double* __restrict__ cv)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int r0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32;
+    if (r0 >= m) return;
+    const int r = r0 + lane;
+    const int n = r < m ? max(cnt[r], 0) : 0, s = r < m ? toff[r] : 0, d = r < m ? crp[r] : 0;
+    // lanes over the entries of the 32 rows together
+    int inc = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(full, inc, o);
+        if (lane >= o) inc += u;
+    }
+    const int total = __shfl_sync(full, inc, 31);
+    for (int f0 = 0; f0 < total; f0 += 32) {
+        const int f = f0 + lane;
+        int k = 0;
+#pragma unroll
+        for (int q = 16; q > 0; q >>= 1)
+            if (__shfl_sync(full, inc, k + q - 1) <= f) k += q;
+        const int before = __shfl_sync(full, inc - n, k), ss = __shfl_sync(full, s, k), dd = __shfl_sync(full, d, k);
+        if (f < total) {
+            cci[dd + f - before] = tci[ss + f - before];
+            cv[dd + f - before] = tv[ss + f - before];
+        }
+    }
+}
+
+// Rows of the overflow list: tables in global memory, one warp each.  The
+// entries of A's row are taken one at a time, in column order, by the whole
+// warp; the lanes share that entry's row of B, whose columns are distinct.
+__global__ void k_gemm_table_size(int nlist, const int* list, const int* prod, int* tsize)
+{
+    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nlist) return;
+    int sz = 1;
+    while (sz < 2 * prod[list[t]]) sz <<= 1;
+    tsize[t] = sz;
+}
+
+__global__ void k_gemm_hash_global(int nlist, const int* list, int row0, const int* arp, const int* aci,
+                                   const double* av, const int* brp, const int* bci, const double* bv,
+                                   const int* toff, int* keys, double* vals, int* cnt, int* run_cnt)
 {
     const int lane = threadIdx.x & 31;
-    const int li = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (li >= m) return;                       // uniform over the warp
-    const int i = row0 + li;
-    const int base = toff[li], size = toff[li + 1] - base;
-    if (size < HASH_WARP_SLOTS) return;
+    const int at = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (at >= nlist) return;                   // uniform over the warp
+    const int i = row0 + list[at];
+    const int base = toff[at], size = toff[at + 1] - base;
     const unsigned mask = (unsigned)size - 1u;
     int c = 0;
     for (int p = arp[i]; p < arp[i + 1]; ++p) {
@@ -632,147 +950,61 @@ __global__ void k_gemm_hash_warp(int m, int row0, const int* arp, const int* aci
         __syncwarp();
     }
     for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
-    if (lane == 0) cnt[li] = c;
+    if (lane == 0) cnt[list[at]] = run_cnt[at] = c;
+}
+
+// Their entries in column order, packed: an entry's rank is the number of
+// smaller columns in its table.
+__global__ void k_gemm_emit_global(const int* toff, const int* keys, const double* vals, const int* crp, int* cci,
+                                   double* cv)
+{
+    const int o = crp[blockIdx.x], t0 = toff[blockIdx.x], t1 = toff[blockIdx.x + 1];
+    for (int t = t0 + threadIdx.x; t < t1; t += blockDim.x) {
+        const int key = keys[t];
+        if (key < 0) continue;
+        int r = 0;
+        for (int q = t0; q < t1; ++q) {
+            const int k = keys[q];
+            r += k >= 0 && k < key;
+        }
+        cci[o + r] = key;
+        cv[o + r] = vals[t];
+    }
+}
+
+// Packed rows src of a list to their places in C, one warp each.
+__global__ void k_gemm_pack_list(int nlist, const int* list, const int* srp, const int* crp, const int* sci,
+                                 const double* sv, int* cci, double* cv)
+{
+    const int lane = threadIdx.x & 31, at = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (at >= nlist) return;
+    const int o = crp[list[at]] - srp[at];
+    for (int t = srp[at] + lane; t < srp[at + 1]; t += 32) {
+        cci[o + t] = sci[t];
+        cv[o + t] = sv[t];
+    }
+}
+
+// overflow rows: empty in the scratch piece
+__global__ void k_gemm_mark(int nlist, const int* list, int* cnt)
+{
+    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < nlist) cnt[list[t]] = 0;
+}
+
+__global__ void k_sum_int(int n, const int* __restrict__ x, unsigned long long* out)
+{
+    unsigned long long s = 0;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        s += (unsigned long long)x[i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0 && s) atomicAdd(out, s);
 }
 
 __global__ void k_shift_rowptr(int m, const int* prp, int off, int* crp)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < m) crp[i] = prp[i] + off;
-}
-
-// Emit of the rows longer than `skip` entries: one thread per row,
-// insertion into column order.
-__global__ void k_gemm_emit(int m, const int* toff, const int* keys, const double* vals,
-                            const int* crp, int* cci, double* cv, int skip)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m || crp[i + 1] - crp[i] <= skip) return;
-    int o = crp[i], s = crp[i];
-    for (int t = toff[i]; t < toff[i + 1]; ++t) {
-        int j = keys[t];
-        if (j < 0) continue;
-        double v = vals[t];
-        int b = o - 1;
-        while (b >= s && cci[b] > j) { cci[b + 1] = cci[b]; cv[b + 1] = cv[b]; --b; }
-        cci[b + 1] = j;
-        cv[b + 1] = v;
-        ++o;
-    }
-}
-
-// Emit of the rows of at most 32 entries: one warp per row, one entry per
-// lane, sorted by column with a bitonic network of warp shuffles.
-__global__ void k_gemm_emit_small(int m, const int* toff, const int* keys, const double* vals,
-                                  const int* crp, int* cci, double* cv)
-{
-    const int lane = threadIdx.x & 31;
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (i >= m) return;                        // uniform over the warp
-    const int n = crp[i + 1] - crp[i];
-    if (n > 32) return;
-    int k = 0x7fffffff;
-    double v = 0.0;
-    int filled = 0;
-    for (int tb = toff[i]; tb < toff[i + 1]; tb += 32) {
-        const int t = tb + lane;
-        const int key = t < toff[i + 1] ? keys[t] : -1;
-        const unsigned ball = __ballot_sync(0xffffffffu, key >= 0);
-        const int pos = filled + __popc(ball & ((1u << lane) - 1u));
-        const double val = key >= 0 ? vals[t] : 0.0;
-        // lane pos receives this entry
-        for (int src = 0; src < 32; ++src) {
-            if (!((ball >> src) & 1u)) continue;
-            const int sp = __shfl_sync(0xffffffffu, pos, src);
-            const int sk = __shfl_sync(0xffffffffu, key, src);
-            const double sv = __shfl_sync(0xffffffffu, val, src);
-            if (lane == sp) { k = sk; v = sv; }
-        }
-        filled += __popc(ball);
-    }
-    for (int size = 2; size <= 32; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            const int ok = __shfl_xor_sync(0xffffffffu, k, stride);
-            const double ov = __shfl_xor_sync(0xffffffffu, v, stride);
-            const bool lower = (lane & stride) == 0;
-            const bool up = (lane & size) == 0;
-            // the lower lane of a pair keeps the smaller key when sorting up
-            const bool take = lower == up ? ok < k : ok > k;
-            if (take) { k = ok; v = ov; }
-        }
-    }
-    if (lane < n) {
-        cci[crp[i] + lane] = k;
-        cv[crp[i] + lane] = v;
-    }
-}
-
-// Emit of the rows of at most EMIT_CAP entries: one warp per row takes the
-// valid slots of the row's table into shared memory (ballot / prefix
-// count), sorts them by column with a bitonic network and writes them out.
-// The values were summed in the hash phase; only their order is set here.
-constexpr int EMIT_CAP = 1024;
-constexpr int EMIT_WARPS = 4;
-
-__global__ void __launch_bounds__(EMIT_WARPS * 32)
-k_gemm_emit_warp(int m, const int* toff, const int* keys, const double* vals, const int* crp, int* cci,
-                 double* cv)
-{
-    __shared__ int sk[EMIT_WARPS][EMIT_CAP];
-    __shared__ double sv[EMIT_WARPS][EMIT_CAP];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int i = blockIdx.x * EMIT_WARPS + w;
-    if (i >= m) return;
-    const int n = crp[i + 1] - crp[i];
-    if (n > EMIT_CAP || n <= 32) return;
-    int* k = sk[w];
-    double* v = sv[w];
-    const int t0 = toff[i], t1 = toff[i + 1];
-    int filled = 0;
-    for (int tb = t0; tb < t1; tb += 32) {
-        const int t = tb + lane;
-        const int key = t < t1 ? keys[t] : -1;
-        const unsigned ball = __ballot_sync(0xffffffffu, key >= 0);
-        if (key >= 0) {
-            const int pos = filled + __popc(ball & ((1u << lane) - 1u));
-            if (pos < EMIT_CAP) {
-                k[pos] = key;
-                v[pos] = vals[t];
-            }
-        }
-        filled += __popc(ball);
-    }
-    int P = 1;
-    while (P < n) P <<= 1;
-    for (int t = n + lane; t < P; t += 32) {
-        k[t] = 0x7fffffff;
-        v[t] = 0.0;
-    }
-    __syncwarp();
-    for (int size = 2; size <= P; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int t = lane; t < P; t += 32) {
-                const int u = t ^ stride;
-                if (u > t) {
-                    const bool up = (t & size) == 0;
-                    const int a = k[t], b = k[u];
-                    if ((a > b) == up && a != b) {
-                        k[t] = b;
-                        k[u] = a;
-                        const double x = v[t];
-                        v[t] = v[u];
-                        v[u] = x;
-                    }
-                }
-            }
-            __syncwarp();
-        }
-    }
-    const int o = crp[i];
-    for (int t = lane; t < n; t += 32) {
-        cci[o + t] = k[t];
-        cv[o + t] = v[t];
-    }
 }
 
 // ------------------------------------------------------------ drop rules --
@@ -1007,71 +1239,145 @@ void submatrix(const DevCSR& A, const int* rows, int nr, const int* colmap, int 
     CK_LAUNCH();
 }
 
-// C = A B.  Rows are processed in chunks whose hash tables hold at most
-// 2^28 slots (3 GiB) together, so large fill-heavy levels neither overflow
-// the int32 table offsets nor exhaust memory; each chunk's rows are emitted
-// into a piece that is then copied into C.
+// Rows [r0, r1) of C = A B as a piece of its own (packed).  prod, room: the
+// rows' products and scratch entries.
+struct GemmPiece {
+    int r0 = 0, r1 = 0, nnz = 0;
+    DBuf<int> rp, ci;
+    DBuf<double> v;
+};
+
+void gemm_piece(const DevCSR& A, const DevCSR& B, const int* prod, const int* room, long long limit, GemmPiece& P,
+                cudaStream_t st)
+{
+    const int mc = P.r1 - P.r0;
+    DBuf<int> toff(size_t(mc) + 1);
+    const int nroom = mc ? exclusive_scan(room, toff.p, mc, st) : 0;
+    DBuf<int> tci(size_t(std::max(nroom, 1)));
+    DBuf<double> tv(size_t(std::max(nroom, 1)));
+    DBuf<int> lists(4 * size_t(std::max(mc, 1))), over(size_t(std::max(mc, 1))), counts(8), cnt(size_t(mc) + 1);
+    CK(cudaMemsetAsync(counts.p, 0, counts.bytes(), st));
+    if (mc) k_gemm_lists<<<grid_for(mc, TB), TB, 0, st>>>(mc, prod, lists.p, counts.p, cnt.p);
+    CK_LAUNCH();
+    int nc[4];
+    d2h(nc, counts.p, 4, st);
+    auto list = [&](int c) { return lists.p + size_t(c) * size_t(mc); };
+    if (nc[0])
+        k_gemm_lanes<GEMM_TINY><<<grid_for(nc[0], TB / GEMM_TINY), TB, 0, st>>>(
+            nc[0], list(0), P.r0, A.rp.p, A.ci.p, A.v.p, B.rp.p, B.ci.p, B.v.p, toff.p, tci.p, tv.p, cnt.p);
+    if (nc[1])
+        k_gemm_lanes<GEMM_SMALL><<<grid_for(nc[1], TB / GEMM_SMALL), TB, 0, st>>>(
+            nc[1], list(1), P.r0, A.rp.p, A.ci.p, A.v.p, B.rp.p, B.ci.p, B.v.p, toff.p, tci.p, tv.p, cnt.p);
+    auto hash = [&](auto kernel, int slots, int c) {
+        if (!nc[c]) return;
+        CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(gemm_smem(slots))));
+        kernel<<<grid_for(nc[c], GEMM_WARPS), GEMM_WARPS * 32, gemm_smem(slots), st>>>(
+            nc[c], list(c), P.r0, A.rp.p, A.ci.p, A.v.p, B.rp.p, B.ci.p, B.v.p, prod, toff.p, tci.p, tv.p, cnt.p,
+            over.p, counts.p + 4);
+    };
+    hash(k_gemm_hash<GEMM_SLOTS_LOW>, GEMM_SLOTS_LOW, 2);
+    hash(k_gemm_hash<GEMM_SLOTS>, GEMM_SLOTS, 3);
+    CK_LAUNCH();
+    // rows beyond the shared-memory tables, in runs whose tables hold at most
+    // `limit` slots together (a row's own table may be larger); each run's
+    // sorted rows wait in a piece of their own until the row pointers stand
+    struct Run {
+        int first = 0, n = 0;
+        DBuf<int> rp, ci;
+        DBuf<double> v;
+    };
+    std::vector<Run> runs;
+    const int nover = nc[3] ? read1(counts.p + 4, st) : 0;
+    if (nover) {
+        DBuf<int> tsize(static_cast<size_t>(nover));
+        k_gemm_table_size<<<grid_for(nover, TB), TB, 0, st>>>(nover, over.p, prod, tsize.p);
+        CK_LAUNCH();
+        std::vector<int> ts(static_cast<size_t>(nover));
+        d2h(ts.data(), tsize.p, size_t(nover), st);
+        for (int t0 = 0; t0 < nover;) {
+            Run R;
+            R.first = t0;
+            long long slots = 0;
+            while (t0 < nover && (t0 == R.first || slots + ts[t0] <= limit)) slots += ts[t0++];
+            R.n = t0 - R.first;
+            const int* rows = over.p + R.first;
+            DBuf<int> gtoff(size_t(R.n) + 1), keys;
+            DBuf<double> vals;
+            CK(cudaMemcpyAsync(gtoff.p, tsize.p + R.first, size_t(R.n) * sizeof(int), cudaMemcpyDeviceToDevice, st));
+            const int total = exclusive_scan(gtoff.p, gtoff.p, R.n, st);
+            keys.alloc(size_t(total));
+            vals.alloc(size_t(total));
+            CK(cudaMemsetAsync(keys.p, 0xff, keys.bytes(), st));
+            R.rp.alloc(size_t(R.n) + 1);
+            k_gemm_hash_global<<<grid_for(R.n, TB / 32), TB, 0, st>>>(R.n, rows, P.r0, A.rp.p, A.ci.p, A.v.p, B.rp.p,
+                                                                     B.ci.p, B.v.p, gtoff.p, keys.p, vals.p, cnt.p,
+                                                                     R.rp.p);
+            CK_LAUNCH();
+            const int n = exclusive_scan(R.rp.p, R.rp.p, R.n, st);
+            R.ci.alloc(size_t(std::max(n, 1)));
+            R.v.alloc(size_t(std::max(n, 1)));
+            k_gemm_emit_global<<<R.n, TB, 0, st>>>(gtoff.p, keys.p, vals.p, R.rp.p, R.ci.p, R.v.p);
+            CK_LAUNCH();
+            CK(cudaStreamSynchronize(st));   // the tables are released
+            runs.push_back(std::move(R));
+        }
+    }
+    P.rp.alloc(size_t(mc) + 1);
+    P.nnz = exclusive_scan(cnt.p, P.rp.p, mc, st);
+    if (nover) {   // nothing of theirs is in the scratch piece
+        k_gemm_mark<<<grid_for(nover, TB), TB, 0, st>>>(nover, over.p, cnt.p);
+        CK_LAUNCH();
+    }
+    P.ci.alloc(std::max(P.nnz, 1));
+    P.v.alloc(std::max(P.nnz, 1));
+    if (mc)
+        k_gemm_pack<<<grid_for(mc, TB), TB, 0, st>>>(mc, toff.p, P.rp.p, cnt.p, tci.p, tv.p, P.ci.p, P.v.p);
+    for (const Run& R : runs)
+        k_gemm_pack_list<<<grid_for(R.n, TB / 32), TB, 0, st>>>(R.n, over.p + R.first, R.rp.p, P.rp.p, R.ci.p, R.v.p,
+                                                               P.ci.p, P.v.p);
+    CK_LAUNCH();
+    CK(cudaStreamSynchronize(st));   // the scratch is released on return
+}
+
+// C = A B.  Rows are processed in pieces whose scratch rows hold at most
+// 2^28 entries (3 GiB) together, so large fill-heavy levels neither overflow
+// the int32 offsets nor exhaust memory; the pieces are then joined.
 void spgemm(const DevCSR& A, const DevCSR& B, DevCSR& C, cudaStream_t st)
 {
     int m = A.n_rows;
     C.n_rows = m;
     C.n_cols = B.n_cols;
-    DBuf<int> tsize(size_t(m) + 1);
-    if (m) k_gemm_bound<<<grid_for(m, TB), TB, 0, st>>>(m, A.rp.p, A.ci.p, B.rp.p, tsize.p);
-    CK_LAUNCH();
-    std::vector<int> ts(static_cast<size_t>(m));
-    d2h(ts.data(), tsize.p, size_t(m), st);
     static long long kLimit = 0;
     if (!kLimit) {
         const char* e = getenv("AIRG_SPGEMM_SLOTS");   // tuning / testing override
         kLimit = e ? std::max(1LL, atoll(e)) : (1LL << 28);
     }
+    DBuf<int> prod(size_t(std::max(m, 1))), room(size_t(std::max(m, 1)));
+    DBuf<unsigned long long> sum(1);
+    CK(cudaMemsetAsync(sum.p, 0, sizeof(unsigned long long), st));
+    if (m) {
+        k_gemm_bound<<<grid_for(m, TB), TB, 0, st>>>(m, 0, A.rp.p, A.ci.p, B.rp.p, prod.p, room.p);
+        k_sum_int<<<std::min(grid_for(m, TB), 1024), TB, 0, st>>>(m, room.p, sum.p);
+    }
+    CK_LAUNCH();
     std::vector<int> cut{0};
-    long long acc = 0;
-    for (int i = 0; i < m; ++i) {
-        if (acc + ts[i] > kLimit && i > cut.back()) { cut.push_back(i); acc = 0; }
-        acc += ts[i];
+    if ((long long)read1(sum.p, st) > kLimit) {
+        std::vector<int> rm(static_cast<size_t>(m));
+        d2h(rm.data(), room.p, size_t(m), st);
+        long long acc = 0;
+        for (int i = 0; i < m; ++i) {
+            if (acc + rm[i] > kLimit && i > cut.back()) { cut.push_back(i); acc = 0; }
+            acc += rm[i];
+        }
     }
     cut.push_back(m);
-    struct Piece {
-        int r0 = 0, r1 = 0, nnz = 0;
-        DBuf<int> rp, ci;
-        DBuf<double> v;
-    };
-    std::vector<Piece> pieces;
+    std::vector<GemmPiece> pieces;
     long long total = 0;
     for (size_t c = 0; c + 1 < cut.size(); ++c) {
-        Piece P;
+        GemmPiece P;
         P.r0 = cut[c];
         P.r1 = cut[c + 1];
-        int mc = P.r1 - P.r0;
-        DBuf<int> toff(size_t(mc) + 1);
-        if (mc) CK(cudaMemcpyAsync(toff.p, tsize.p + P.r0, size_t(mc) * sizeof(int), cudaMemcpyDeviceToDevice, st));
-        int tsz = exclusive_scan(toff.p, toff.p, mc, st);
-        DBuf<int> keys(std::max(tsz, 1));
-        DBuf<double> vals(std::max(tsz, 1));
-        CK(cudaMemsetAsync(keys.p, 0xff, keys.bytes(), st));
-        P.rp.alloc(size_t(mc) + 1);
-        if (mc) {
-            k_gemm_hash<<<grid_for(mc, TB), TB, 0, st>>>(mc, P.r0, A.rp.p, A.ci.p, A.v.p, B.rp.p, B.ci.p,
-                                                         B.v.p, toff.p, keys.p, vals.p, P.rp.p);
-            k_gemm_hash_warp<<<grid_for(mc, TB / 32), TB, 0, st>>>(mc, P.r0, A.rp.p, A.ci.p, A.v.p, B.rp.p,
-                                                                   B.ci.p, B.v.p, toff.p, keys.p, vals.p, P.rp.p);
-        }
-        CK_LAUNCH();
-        P.nnz = exclusive_scan(P.rp.p, P.rp.p, mc, st);
-        P.ci.alloc(std::max(P.nnz, 1));
-        P.v.alloc(std::max(P.nnz, 1));
-        if (mc) {
-            k_gemm_emit_small<<<grid_for(mc, TB / 32), TB, 0, st>>>(mc, toff.p, keys.p, vals.p, P.rp.p,
-                                                                     P.ci.p, P.v.p);
-            k_gemm_emit_warp<<<grid_for(mc, EMIT_WARPS), EMIT_WARPS * 32, 0, st>>>(mc, toff.p, keys.p, vals.p,
-                                                                                   P.rp.p, P.ci.p, P.v.p);
-            k_gemm_emit<<<grid_for(mc, TB), TB, 0, st>>>(mc, toff.p, keys.p, vals.p, P.rp.p, P.ci.p, P.v.p,
-                                                         EMIT_CAP);
-        }
-        CK_LAUNCH();
-        CK(cudaStreamSynchronize(st));
+        gemm_piece(A, B, prod.p + P.r0, room.p + P.r0, kLimit, P, st);
         total += P.nnz;
         pieces.push_back(std::move(P));
     }
@@ -1087,7 +1393,7 @@ void spgemm(const DevCSR& A, const DevCSR& B, DevCSR& C, cudaStream_t st)
     C.ci.alloc(std::max(C.nnz, 1));
     C.v.alloc(std::max(C.nnz, 1));
     int off = 0;
-    for (Piece& P : pieces) {
+    for (GemmPiece& P : pieces) {
         int mc = P.r1 - P.r0;
         if (mc) k_shift_rowptr<<<grid_for(mc, TB), TB, 0, st>>>(mc, P.rp.p, off, C.rp.p + P.r0);
         CK_LAUNCH();
