@@ -1159,6 +1159,12 @@ struct Ctx {
     DBuf<unsigned> xticket;          // last-block ticket of k_xdot
     long long ndots = 0;             // exact dot products launched
     HBuf<double> hcol;               // one Hessenberg column on the host
+    // grid state of k_mgs_column: accumulators, [arrivals, error], and what
+    // earlier launches left there
+    DBuf<unsigned long long> cdig;
+    DBuf<unsigned> cbar;
+    unsigned cbase = 0;
+    int cphase = 0;
     explicit Ctx(cudaStream_t s) : st(s)
     {
         xacc.alloc(XD_DIGITS);
@@ -1167,6 +1173,10 @@ struct Ctx {
         CK(cudaMemsetAsync(xacc.p, 0, xacc.bytes(), st));
         CK(cudaMemsetAsync(xbad.p, 0, xbad.bytes(), st));
         CK(cudaMemsetAsync(xticket.p, 0, xticket.bytes(), st));
+        cdig.alloc(3 * XD_DIGITS);
+        cbar.alloc(2);
+        CK(cudaMemsetAsync(cdig.p, 0, cdig.bytes(), st));
+        CK(cudaMemsetAsync(cbar.p, 0, cbar.bytes(), st));
     }
 };
 
@@ -1199,6 +1209,47 @@ void mgs_xdot(Ctx& c, long long n, double* w, const double* vprev, const double*
                                                out_sqrt);
     CK_LAUNCH();
     ++c.ndots;
+}
+
+// Column j of the Gram-Schmidt process of w (length n) against v_0 .. v_j,
+// one launch; false where a row's worth of registers per SM does not hold w.
+// Few elements a thread as long as blocks are left: a block's share of the
+// integer work is ~0.25 us per element and thread, another block adds little
+// to the barrier; up to 2048 elements one block has no barrier at all.
+bool mgs_column(Ctx& c, long long n, const double* V, int j, const double* w, double* vnext, double* hcol)
+{
+    const long long per = XC_THREADS, sms = num_sms();
+    int E = 1;
+    long long grid = 1;
+    if (n <= 4 * per) E = 4;
+    else {
+        while (E < XC_MAX_E && (n + per * E - 1) / (per * E) > sms) E *= 2;
+        grid = (n + per * E - 1) / (per * E);
+    }
+    if (grid > sms || grid < 1) return false;
+    auto launch = [&](auto kernel) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(unsigned(grid));
+        cfg.blockDim = dim3(XC_THREADS);
+        cfg.stream = c.st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = grid > 1 ? 1 : 0;
+        CK(cudaLaunchKernelEx(&cfg, kernel, int(n), V, j, w, vnext, hcol, c.cdig.p, c.cphase, c.cbar.p, c.cbase,
+                              c.xbad.p, reinterpret_cast<int*>(c.cbar.p + 1)));
+    };
+    if (E == 1) launch(k_mgs_column<1>);
+    else if (E == 2) launch(k_mgs_column<2>);
+    else if (E == 4) launch(k_mgs_column<4>);
+    else launch(k_mgs_column<8>);
+    c.ndots += j + 2;
+    if (grid > 1) {
+        c.cbase += unsigned(grid) * unsigned(j + 2);
+        c.cphase = (c.cphase + j + 2) % 3;
+    }
+    return true;
 }
 
 // Wall time of one setup phase, added to *acc: the stream is synchronised
@@ -1465,15 +1516,18 @@ ArnoldiOut arnoldi(Ctx& c, const DevCSR& A, const double* b, int m, double tol, 
     for (int j = 0; j < m; ++j) {
         k_spmv_det<<<grid_for(n, TB), TB, 0, st>>>(int(n), A.rp.p, A.ci.p, A.v.p, V.p + size_t(j) * n, w.p);
         CK_LAUNCH();
-        double* hj = Hd.p + size_t(j) * (m + 1);
         // h_ij = <w, v_i> then w -= h_ij v_i, for i = 0..j (modified
-        // Gram-Schmidt); each update is fused with the next dot product
-        for (int i = 0; i <= j; ++i) {
-            mgs_xdot(c, n, w.p, i ? V.p + size_t(i - 1) * n : nullptr, i ? hj + i - 1 : nullptr,
-                     V.p + size_t(i) * n, hj + i, nullptr);
-        }
+        // Gram-Schmidt), and v_{j+1} = w / ||w||: in one launch where w fits
+        // in registers, else one per dot (each update fused with the next)
+        double* hj = Hd.p + size_t(j) * (m + 1);
         double* hn = hj + j + 1;
-        mgs_xdot(c, n, w.p, V.p + size_t(j) * n, hj + j, nullptr, nullptr, hn);
+        const bool column = mgs_column(c, n, V.p, j, w.p, V.p + size_t(j + 1) * n, hj);
+        if (!column) {
+            for (int i = 0; i <= j; ++i)
+                mgs_xdot(c, n, w.p, i ? V.p + size_t(i - 1) * n : nullptr, i ? hj + i - 1 : nullptr,
+                         V.p + size_t(i) * n, hj + i, nullptr);
+            mgs_xdot(c, n, w.p, V.p + size_t(j) * n, hj + j, nullptr, nullptr, hn);
+        }
         d2h(c.hcol.p, hj, size_t(j) + 2, st);
         for (int i = 0; i <= j + 1; ++i) Hh[size_t(i) * m + j] = col[i];
         double s = 0.0;
@@ -1494,11 +1548,12 @@ ArnoldiOut arnoldi(Ctx& c, const DevCSR& A, const double* b, int m, double tol, 
                 break;
             }
         }
-        if (j + 1 < m) {
+        if (j + 1 < m && !column) {
             k_div_dev<<<g, TB, 0, st>>>(n, V.p + size_t(j + 1) * n, w.p, hn);
             CK_LAUNCH();
         }
     }
+    if (read1(c.cbar.p + 1, st)) fail(AIRG_ERR_TIMEOUT, "a grid barrier of the Gram-Schmidt kernel gave up waiting");
     out.beta = beta_h;
     int k = out.k;
     out.H.assign(size_t(k + 1) * k, 0.0);
