@@ -128,10 +128,11 @@ __device__ __forceinline__ void xd_win_add(unsigned long long* acc, XdWin& a, do
     const int pos = ex + ey + XD_BIAS;
     const int d = pos >> 5;
     if (d != a.d0 && d != a.d0 + 1) {
-        // the window moves so that it holds this digit and, where the
-        // products grew, the one below
+        // the window moves so that it holds this digit and the neighbour
+        // that the product is nearer to: products within 16 bits of this one
+        // need no further move (each is seven shared-memory atomics)
         xd_win_deposit(acc, a);
-        const int d0 = d > a.d0 && d > 0 ? d - 1 : d;
+        const int d0 = (pos & 31) < 16 && d > 0 ? d - 1 : d;
         xd_win_init(a);
         a.d0 = d0;
     }
