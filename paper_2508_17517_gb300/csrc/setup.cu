@@ -330,18 +330,28 @@ __global__ void k_state_to_f(int n, const int8_t* state, int8_t* is_f)
 __global__ void k_ddc_ratio(int n, const int* rp, const int* ci, const double* v,
                             const int8_t* is_f, double* ratio, unsigned long long* rmax_bits)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (!is_f[i]) { ratio[i] = -1.0; return; }
-    double s = 0.0, d = 0.0;
-    for (int k = rp[i]; k < rp[i + 1]; ++k) {
-        int j = ci[k];
-        if (j == i) d = fabs(v[k]);
-        else if (is_f[j]) s = __dadd_rn(s, fabs(v[k]));
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned long long m = 0ULL;
+    if (i < n && !is_f[i]) ratio[i] = -1.0;
+    else if (i < n) {
+        double s = 0.0, d = 0.0;
+        for (int k = rp[i]; k < rp[i + 1]; ++k) {
+            int j = ci[k];
+            if (j == i) d = fabs(v[k]);
+            else if (is_f[j]) s = __dadd_rn(s, fabs(v[k]));
+        }
+        const double r = d > 0.0 ? __ddiv_rn(s, d) : __longlong_as_double(0x7ff0000000000000LL);
+        ratio[i] = r;
+        m = (unsigned long long)__double_as_longlong(r);   // r >= 0: its bits order like its value
     }
-    double r = d > 0.0 ? __ddiv_rn(s, d) : __longlong_as_double(0x7ff0000000000000LL);
-    ratio[i] = r;
-    atomicMax(rmax_bits, (unsigned long long)__double_as_longlong(r));   // r >= 0
+    // one atomic for a warp's rows, and only where it raises the maximum: an
+    // atomic per row on one address serialises the grid (1.2 ms a call on
+    // average over the levels of 4096^2)
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long u = __shfl_xor_sync(0xffffffffu, m, o);
+        m = u > m ? u : m;
+    }
+    if ((threadIdx.x & 31) == 0 && m > *(volatile unsigned long long*)rmax_bits) atomicMax(rmax_bits, m);
 }
 
 __global__ void k_ddc_bin(int n, const int8_t* is_f, const double* ratio, double rmax, int nbins,
@@ -1056,6 +1066,100 @@ __global__ void k_drop_lump(int n, const int* rp, const int* ci, const double* v
     cnt[i] = c;
 }
 
+// The three row kernels above and below for rows of more than a few entries:
+// one warp per row, adjacent lanes on adjacent entries, with the same
+// decisions and the same order of the sums.
+__global__ void k_drop_rows_warp(int n, const int* __restrict__ rp, const double* __restrict__ v, double tol,
+                                 int8_t* __restrict__ keep, int* __restrict__ cnt)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= n) return;
+    const int b = rp[i], e = rp[i + 1];
+    double m = 0.0;
+    for (int k = b + lane; k < e; k += 32)
+        if (fabs(v[k]) > m) m = fabs(v[k]);
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(full, m, o));
+    const double thr = __dmul_rn(tol, m);
+    int c = 0;
+    for (int k0 = b; k0 < e; k0 += 32) {
+        const int k = k0 + lane;
+        const double x = k < e ? v[k] : 0.0;
+        const bool kp = x != 0.0 && fabs(x) >= thr;
+        if (k < e) keep[k] = (int8_t)kp;
+        c += __popc(__ballot_sync(full, kp));
+    }
+    if (lane == 0) cnt[i] = c;
+}
+
+__global__ void k_drop_lump_warp(int n, const int* __restrict__ rp, const int* __restrict__ ci,
+                                 const double* __restrict__ v, double tol, int lump, int8_t* __restrict__ keep,
+                                 double* __restrict__ vout, int* __restrict__ cnt, int* bad)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= n) return;
+    const int b = rp[i], e = rp[i + 1];
+    double m = 0.0;
+    int dpos = -1;
+    for (int k = b + lane; k < e; k += 32) {
+        if (ci[k] == i) dpos = k;
+        else if (fabs(v[k]) > m) m = fabs(v[k]);
+    }
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(full, m, o));
+    dpos = __reduce_max_sync(full, dpos);
+    if (dpos < 0) {
+        if (lane == 0) {
+            *bad = 1;
+            cnt[i] = 0;
+        }
+        return;
+    }
+    const double thr = __dmul_rn(tol, m);
+    double d = v[dpos];
+    int c = 0;
+    for (int k0 = b; k0 < e; k0 += 32) {
+        const int k = k0 + lane;
+        const bool in = k < e;
+        const double x = in ? v[k] : 0.0;
+        const bool drop = in && k != dpos && (x == 0.0 || fabs(x) < thr);
+        if (in) {
+            keep[k] = (int8_t)!drop;
+            if (k != dpos) vout[k] = x;
+        }
+        c += __popc(__ballot_sync(full, in && !drop));
+        if (lump)
+            for (unsigned left = __ballot_sync(full, drop); left; left &= left - 1u)
+                d = __dadd_rn(d, __shfl_sync(full, x, __ffs(left) - 1));
+    }
+    if (lane == 0) {
+        vout[dpos] = d;
+        cnt[i] = c;
+    }
+}
+
+__global__ void k_compact_warp(int n, const int* __restrict__ rp, const int* __restrict__ ci,
+                               const double* __restrict__ v, const int8_t* __restrict__ keep,
+                               const int* __restrict__ nrp, int* __restrict__ nci, double* __restrict__ nv)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= n) return;
+    const int b = rp[i], e = rp[i + 1];
+    int o = nrp[i];
+    for (int k0 = b; k0 < e; k0 += 32) {
+        const int k = k0 + lane;
+        const bool kp = k < e && keep[k];
+        const unsigned on = __ballot_sync(full, kp);
+        if (kp) {
+            const int at = o + __popc(on & ((1u << lane) - 1u));
+            nci[at] = ci[k];
+            nv[at] = v[k];
+        }
+        o += __popc(on);
+    }
+}
+
 __global__ void k_compact(int n, const int* rp, const int* ci, const double* v,
                           const int8_t* keep, const int* nrp, int* nci, double* nv)
 {
@@ -1458,6 +1562,12 @@ void spgemm(const DevCSR& A, const DevCSR& B, DevCSR& C, cudaStream_t st)
     CK(cudaStreamSynchronize(st));
 }
 
+// Rows of more than 8 entries on average take the row kernels with a warp per
+// row: with one thread per row the 32 rows of a warp are that far apart in
+// memory.  Drop and lumping of the 4096^2 setup with its compaction: 55 ->
+// 30 ms.
+bool long_rows(const DevCSR& A) { return A.n_rows > 0 && A.nnz > 8LL * A.n_rows; }
+
 void compact(const DevCSR& A, const int8_t* keep, DBuf<int>& cnt, DevCSR& out, cudaStream_t st)
 {
     int n = A.n_rows;
@@ -1467,8 +1577,11 @@ void compact(const DevCSR& A, const int8_t* keep, DBuf<int>& cnt, DevCSR& out, c
     out.nnz = counts_to_rowptr(out.rp, n, st);
     out.ci.alloc(out.nnz);
     out.v.alloc(out.nnz);
-    if (n) k_compact<<<grid_for(n, TB), TB, 0, st>>>(n, A.rp.p, A.ci.p, A.v.p, keep, out.rp.p,
-                                                       out.ci.p, out.v.p);
+    if (long_rows(A))
+        k_compact_warp<<<grid_for(n, TB / 32), TB, 0, st>>>(n, A.rp.p, A.ci.p, A.v.p, keep, out.rp.p, out.ci.p,
+                                                            out.v.p);
+    else if (n)
+        k_compact<<<grid_for(n, TB), TB, 0, st>>>(n, A.rp.p, A.ci.p, A.v.p, keep, out.rp.p, out.ci.p, out.v.p);
     CK_LAUNCH();
 }
 
@@ -1974,8 +2087,12 @@ std::unique_ptr<Hierarchy> build_hierarchy(DevCSR&& A0, const airg_options& o, c
             if (Zfull.nnz) k_scale<<<grid_for(Zfull.nnz, TB), TB, 0, st>>>(Zfull.nnz, Zfull.v.p, -1.0);
             DBuf<int8_t> keep(std::max(Zfull.nnz, 1));
             DBuf<int> cnt(size_t(L->n_c) + 1);
-            if (L->n_c) k_drop_rows<<<grid_for(L->n_c, TB), TB, 0, st>>>(L->n_c, Zfull.rp.p, Zfull.v.p,
-                                                                         o.r_drop, keep.p, cnt.p);
+            if (long_rows(Zfull))
+                k_drop_rows_warp<<<grid_for(L->n_c, TB / 32), TB, 0, st>>>(L->n_c, Zfull.rp.p, Zfull.v.p, o.r_drop,
+                                                                           keep.p, cnt.p);
+            else if (L->n_c)
+                k_drop_rows<<<grid_for(L->n_c, TB), TB, 0, st>>>(L->n_c, Zfull.rp.p, Zfull.v.p, o.r_drop, keep.p,
+                                                                 cnt.p);
             CK_LAUNCH();
             compact(Zfull, keep.p, cnt, L->Z, st);
         }
@@ -2024,8 +2141,12 @@ std::unique_ptr<Hierarchy> build_hierarchy(DevCSR&& A0, const airg_options& o, c
             DBuf<double> vout(std::max(Ac.nnz, 1));
             DBuf<int> cnt(size_t(nc) + 1), bad(1);
             CK(cudaMemsetAsync(bad.p, 0, sizeof(int), st));
-            if (nc) k_drop_lump<<<grid_for(nc, TB), TB, 0, st>>>(nc, Ac.rp.p, Ac.ci.p, Ac.v.p, o.a_drop,
-                                                                o.a_lump, keep.p, vout.p, cnt.p, bad.p);
+            if (long_rows(Ac))
+                k_drop_lump_warp<<<grid_for(nc, TB / 32), TB, 0, st>>>(nc, Ac.rp.p, Ac.ci.p, Ac.v.p, o.a_drop, o.a_lump,
+                                                                       keep.p, vout.p, cnt.p, bad.p);
+            else if (nc)
+                k_drop_lump<<<grid_for(nc, TB), TB, 0, st>>>(nc, Ac.rp.p, Ac.ci.p, Ac.v.p, o.a_drop, o.a_lump, keep.p,
+                                                             vout.p, cnt.p, bad.p);
             CK_LAUNCH();
             if (read1(bad.p, st)) fail(AIRG_ERR_BREAKDOWN, "coarse row without a diagonal");
             std::swap(Ac.v.p, vout.p);
