@@ -63,6 +63,14 @@ __global__ void k_sell_width(int nrows, int nslices, const int* rp, const int* c
     width[s] = w * 32;
 }
 
+// *out = the largest of the slices' slots (32 x entries)
+__global__ void k_sell_widest(int nslices, const int* __restrict__ width, int* out)
+{
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    const int m = __reduce_max_sync(0xffffffffu, s < nslices ? width[s] : 0);
+    if ((threadIdx.x & 31) == 0 && m > *(volatile int*)out) atomicMax(out, m);
+}
+
 template <class T>
 __global__ void k_sell_fill(int nrows, int nslices, const int* rp, const int* ci, const double* v,
                             const int* src_row, const int* cmap, const int* sptr, int* col, T* val,
@@ -137,11 +145,13 @@ void build_sell(const DevCSR& A, const int* src_row, const int* cmap, int n_cols
         k_sell_width<<<grid_for(S.n_slices, TB), TB, 0, st>>>(A.n_rows, S.n_slices, A.rp.p, A.ci.p, src_row,
                                                                 cmap, split_diag ? 1 : 0, S.sptr.p);
     CK_LAUNCH();
+    DBuf<unsigned long long> cnt(2);
+    CK(cudaMemsetAsync(cnt.p, 0, cnt.bytes(), st));
+    if (S.n_slices)
+        k_sell_widest<<<grid_for(S.n_slices, TB), TB, 0, st>>>(S.n_slices, S.sptr.p, reinterpret_cast<int*>(cnt.p + 1));
     S.padded = exclusive_scan(S.sptr.p, S.sptr.p, S.n_slices, st);
     S.col.alloc(std::max<long long>(S.padded, 1));
     S.val.alloc(std::max<long long>(S.padded, 1));
-    DBuf<unsigned long long> cnt(1);
-    CK(cudaMemsetAsync(cnt.p, 0, sizeof(unsigned long long), st));
     if (split_diag) S.diag.alloc(std::max(A.n_rows, 1));
     if (S.n_slices)
         k_sell_fill<T><<<grid_for((long long)S.n_slices * 32, TB), TB, 0, st>>>(
@@ -149,9 +159,10 @@ void build_sell(const DevCSR& A, const int* src_row, const int* cmap, int n_cols
             split_diag ? S.diag.p : nullptr, cnt.p);
     if (S.n_slices) k_sell_pad<<<grid_for((long long)S.n_slices * 32, TB), TB, 0, st>>>(S.n_slices, S.sptr.p, S.col.p);
     CK_LAUNCH();
-    unsigned long long nd = 0;
-    d2h(&nd, cnt.p, 1, st);
-    S.ndiag = (long long)nd;
+    unsigned long long nd[2] = {0, 0};
+    d2h(nd, cnt.p, 2, st);
+    S.ndiag = (long long)nd[0];
+    S.mw = int(nd[1] >> 5);
     if (!split_diag) S.diag = DBuf<T>();
 }
 
@@ -252,6 +263,7 @@ void copy_sell_bf16(const Sell<double>& S, Sell<float, bf16s>& out, cudaStream_t
     out.n_slices = S.n_slices;
     out.k = S.k;
     out.r = S.r;
+    out.mw = S.mw;
     out.nnz = S.nnz;
     out.padded = S.padded;
     out.ndiag = 0;
@@ -271,6 +283,7 @@ void copy_sell_f32(const Sell<double>& S, Sell<float>& out, cudaStream_t st)
     out.n_slices = S.n_slices;
     out.k = S.k;
     out.r = S.r;
+    out.mw = S.mw;
     out.nnz = S.nnz;
     out.padded = S.padded;
     out.ndiag = S.ndiag;
@@ -417,14 +430,49 @@ __device__ __forceinline__ T row_dot(const SellView<T, V>& S, int slice, int lan
     return acc;
 }
 
+// G slices of at most MW entries a row each: all loads of the G rows of a
+// lane, then all gathers, then the sums.
+template <class T, int G, int MW, class V, bool C16>
+__device__ __forceinline__ void dot_narrow(const SellView<T, V>& S, const T* __restrict__ x, const int* b,
+                                           const int* w, const int* cb, T* acc)
+{
+    int c[G][MW];
+    T v[G][MW], xv[G][MW];
+#pragma unroll
+    for (int q = 0; q < G; ++q)
+#pragma unroll
+        for (int u = 0; u < MW; ++u) {
+            const bool ok = u < w[q];
+            c[q][u] = ok ? ldcol<C16>(S.col, S.col16, cb[q], b[q] + 32 * u) : 0;
+            v[q][u] = ok ? ldval<T>(S.val + b[q] + 32 * u) : T(0);
+        }
+#pragma unroll
+    for (int q = 0; q < G; ++q)
+#pragma unroll
+        for (int u = 0; u < MW; ++u) xv[q][u] = u < w[q] ? x[c[q][u]] : T(0);
+#pragma unroll
+    for (int q = 0; q < G; ++q)
+#pragma unroll
+        for (int u = 0; u < MW; ++u)
+            if (u < w[q]) acc[q] = fma(v[q][u], xv[q][u], acc[q]);
+}
+
 // Rows 32 s + lane, s = s0 .. s0+R-1, of S times x for one warp (short rows,
 // one warp per slice).  Per row the arithmetic is fixed: start from
 // diag_r x_r (or 0), then add the row's stored entries in slice order with
 // one fused multiply-add each.  It does not depend on R or on which path
 // below runs, so the slices-per-warp choice never changes a result bit.
-// When every slice is at most 4 wide, all loads of the R rows are issued
-// (predicated) before their gathers, and all gathers before the sums.
-template <class T, int R, class V, bool C16 = false>
+// MW = 1, 2: no slice is wider, all loads of the R rows together.  MW = 4:
+// the same where every slice of the warp is at most four wide, else four
+// slots at a time.  MW = 0: eight slots at a time.  The finest levels have
+// one or two entries a row beside the diagonal, and code for four slots a row
+// (~100 instructions a slice) was what bounded them, not their bytes; each
+// width is a kernel of its own because the registers of the widest path would
+// cost the others their warps.  Measured at 4096^2, before and after: smoother
+// term of level 0 (7.3M rows, MW = 1) 92 -> 52 us FP64, 47 -> 32 us FP32;
+// residual of level 0 (MW = 2) 100 -> 84 us FP64; restriction of levels 3 and
+// 4 (8 to 16 slots, MW = 0) 88 -> 76 and 70 -> 62 us FP64.
+template <class T, int R, class V, bool C16, int MW>
 __device__ __forceinline__ void dot_slices(const SellView<T, V>& S, const T* __restrict__ x, int s0, int lane,
                                            T (&acc)[R])
 {
@@ -442,51 +490,39 @@ __device__ __forceinline__ void dot_slices(const SellView<T, V>& S, const T* __r
         const int r = s * 32 + lane;
         acc[q] = (S.diag && r < S.n_rows) ? __ldg(S.diag + r) * x[r] : T(0);
     }
-    if (fits) {
-        int c[R][4];
-        T v[R][4], xv[R][4];
+    if constexpr (MW == 1 || MW == 2) {
+        dot_narrow<T, R, MW, V, C16>(S, x, b, w, cb, acc);
+        return;
+    }
+    if (MW == 4 && fits) {
+        dot_narrow<T, R, 4, V, C16>(S, x, b, w, cb, acc);
+        return;
+    }
+    constexpr int U = MW == 4 ? 4 : 8;
 #pragma unroll
-        for (int q = 0; q < R; ++q)
+    for (int q = 0; q < R; ++q) {
+        for (int u0 = 0; u0 < w[q]; u0 += U) {
+            int c[U];
+            T v[U], xv[U];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const bool ok = u < w[q];
-                c[q][u] = ok ? ldcol<C16>(S.col, S.col16, cb[q], b[q] + 32 * u) : 0;
-                v[q][u] = ok ? ldval<T>(S.val + b[q] + 32 * u) : T(0);
+            for (int u = 0; u < U; ++u) {
+                const bool ok = u0 + u < w[q];
+                c[u] = ok ? ldcol<C16>(S.col, S.col16, cb[q], b[q] + 32 * (u0 + u)) : 0;
+                v[u] = ok ? ldval<T>(S.val + b[q] + 32 * (u0 + u)) : T(0);
             }
 #pragma unroll
-        for (int q = 0; q < R; ++q)
+            for (int u = 0; u < U; ++u) xv[u] = u0 + u < w[q] ? x[c[u]] : T(0);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) xv[q][u] = u < w[q] ? x[c[q][u]] : T(0);
-#pragma unroll
-        for (int q = 0; q < R; ++q)
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (u < w[q]) acc[q] = fma(v[q][u], xv[q][u], acc[q]);
-    } else {
-#pragma unroll
-        for (int q = 0; q < R; ++q) {
-            for (int u0 = 0; u0 < w[q]; u0 += 4) {
-                int c[4];
-                T v[4], xv[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const bool ok = u0 + u < w[q];
-                    c[u] = ok ? ldcol<C16>(S.col, S.col16, cb[q], b[q] + 32 * (u0 + u)) : 0;
-                    v[u] = ok ? ldval<T>(S.val + b[q] + 32 * (u0 + u)) : T(0);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) xv[u] = u0 + u < w[q] ? x[c[u]] : T(0);
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (u0 + u < w[q]) acc[q] = fma(v[u], xv[u], acc[q]);
-            }
+            for (int u = 0; u < U; ++u)
+                if (u0 + u < w[q]) acc[q] = fma(v[u], xv[u], acc[q]);
         }
     }
 }
 
 // Applies epi(r, (S x)_r, pre(r)) to every row r of S.  pre(r) loads the
 // row's other operands; it runs before the row's gathers so that its loads
-// overlap them.  K = warps per slice.  R = slices per warp for K = 1, and
+// overlap them.  K = warps per slice; for one warp per slice K is -1 or -2 (no
+// slice wider than one, two entries), 1 (four on average) or 0 (more).  R = slices per warp for K = 1, and
 // loads in flight per lane (4, 8 or 16) for K > 1; in neither case does R
 // change the arithmetic.
 template <class T, int K, int R, bool C16 = false, class V, class Pre, class Epi>
@@ -500,7 +536,7 @@ __device__ __forceinline__ void for_rows(const SellView<T, V>& S, const T* __res
     // rev != 0 takes the groups of slices in reverse order (block 0 the last
     // group): a chain of steps over one operator that alternates the
     // direction starts each step on the lines the previous one left in L2.
-    if constexpr (K == 1) {
+    if constexpr (K <= 1) {
         const int nw = (gridDim.x * blockDim.x) >> 5;
         const int ngr = (S.n_slices + R - 1) / R;
         for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < ngr; w += nw) {
@@ -512,7 +548,7 @@ __device__ __forceinline__ void for_rows(const SellView<T, V>& S, const T* __res
                 pv[q] = r < S.n_rows ? pre(r) : PV{};
             }
             T acc[R];
-            dot_slices<T, R, V, C16>(S, x, s0, lane, acc);
+            dot_slices<T, R, V, C16, K == 1 ? 4 : -K>(S, x, s0, lane, acc);
 #pragma unroll
             for (int q = 0; q < R; ++q) {
                 const int r = (s0 + q) * 32 + lane;
@@ -813,12 +849,38 @@ inline int grid_rows(const Sell<T, V>& S, F* kernel)
 template <class T, class V>
 inline int block_rows(const Sell<T, V>& S) { return bk(S.k); }
 
-// Runs the statement with compile-time KK (warps per slice) and RR (slices
-// per warp for KK = 1, loads in flight per lane for KK > 1) of operator S.
+// Runs the statement with compile-time KK (warps per slice; for one warp per
+// slice 1, -1, -2 or 0 by the widest slice, see for_rows) and RR (slices per
+// warp for KK <= 1, where one slice of at most two entries is no warp's work
+// by itself; loads in flight per lane for KK > 1) of operator S.
 #define WITH_KR(S, ...)                                                         \
     do {                                                                        \
-        if ((S).k == 1) {                                                       \
+        if ((S).k == 1 && (S).mw <= 1) {                                        \
+            constexpr int KK = -1;                                              \
+            switch ((S).r) {                                                    \
+                case 1: { constexpr int RR = 2; __VA_ARGS__; } break;           \
+                case 2: { constexpr int RR = 2; __VA_ARGS__; } break;           \
+                case 4: { constexpr int RR = 4; __VA_ARGS__; } break;           \
+                default: fail(AIRG_ERR_STATE, "bad slices-per-warp");           \
+            }                                                                   \
+        } else if ((S).k == 1 && (S).mw <= 2) {                                 \
+            constexpr int KK = -2;                                              \
+            switch ((S).r) {                                                    \
+                case 1: { constexpr int RR = 2; __VA_ARGS__; } break;           \
+                case 2: { constexpr int RR = 2; __VA_ARGS__; } break;           \
+                case 4: { constexpr int RR = 4; __VA_ARGS__; } break;           \
+                default: fail(AIRG_ERR_STATE, "bad slices-per-warp");           \
+            }                                                                   \
+        } else if ((S).k == 1 && (S).padded <= 128LL * (S).n_slices) {          \
             constexpr int KK = 1;                                               \
+            switch ((S).r) {                                                    \
+                case 1: { constexpr int RR = 1; __VA_ARGS__; } break;           \
+                case 2: { constexpr int RR = 2; __VA_ARGS__; } break;           \
+                case 4: { constexpr int RR = 4; __VA_ARGS__; } break;           \
+                default: fail(AIRG_ERR_STATE, "bad slices-per-warp");           \
+            }                                                                   \
+        } else if ((S).k == 1) {                                                \
+            constexpr int KK = 0;                                               \
             switch ((S).r) {                                                    \
                 case 1: { constexpr int RR = 1; __VA_ARGS__; } break;           \
                 case 2: { constexpr int RR = 2; __VA_ARGS__; } break;           \

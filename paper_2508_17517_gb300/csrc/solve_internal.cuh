@@ -60,6 +60,7 @@ struct bf16s {
 template <class T, class V = T>
 struct Sell {
     int n_rows = 0, n_cols = 0, n_slices = 0, k = 1, r = 1;
+    int mw = 0;        // entries a row of the widest slice
     int persist = 0;   // 1: row kernels run on a grid of resident blocks that stride over the slices
     int stream = 0;    // coarsest operator only: 1 = its steps stream it through shared memory (coarse_stream.cu)
     int xs = 0;   // coarsest operator only: > 0 = its SpMVs stage x in shared memory, on xs blocks (solve.cu)
@@ -74,7 +75,7 @@ struct Sell {
 
 template <class T, class V = T>
 struct SellView {
-    int n_rows, n_slices;
+    int n_rows, n_slices, mw;
     const int* __restrict__ sptr;
     const int* __restrict__ col;
     const V* __restrict__ val;
@@ -86,7 +87,7 @@ struct SellView {
 template <class T, class V>
 SellView<T, V> view(const Sell<T, V>& s)
 {
-    return SellView<T, V>{s.n_rows, s.n_slices, s.sptr.p, s.col.p, s.val.p, s.ndiag ? s.diag.p : nullptr,
+    return SellView<T, V>{s.n_rows, s.n_slices, s.mw, s.sptr.p, s.col.p, s.val.p, s.ndiag ? s.diag.p : nullptr,
                           s.col16.n ? s.col16.p : nullptr, s.cbase.n ? s.cbase.p : nullptr};
 }
 
