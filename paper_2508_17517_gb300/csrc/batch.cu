@@ -601,7 +601,7 @@ BShape bshape(int k)
     do {                                                                             \
         const BShape bs_ = bshape<T>(k);                                             \
         const int lg = bs_.lg;                                                       \
-        if ((S).k == 1) { constexpr int PW = 1; WITH_SHAPE(T, bs_, __VA_ARGS__); }   \
+        if ((S).pw == 1) { constexpr int PW = 1; WITH_SHAPE(T, bs_, __VA_ARGS__); }  \
         else { constexpr int PW = 4; WITH_SHAPE(T, bs_, __VA_ARGS__); }              \
     } while (0)
 

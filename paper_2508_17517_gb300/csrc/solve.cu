@@ -137,7 +137,8 @@ void build_sell(const DevCSR& A, const int* src_row, const int* cmap, int n_cols
     S.n_rows = A.n_rows;
     S.n_cols = n_cols;
     S.nnz = A.nnz;
-    S.k = choose_parts(A.nnz, A.n_rows);
+    S.k = choose_parts(A.nnz, A.n_rows, true);
+    S.pw = A.n_rows && A.nnz > 12LL * A.n_rows ? 4 : 1;
     S.r = S.k == 1 ? 1 : 4;
     S.n_slices = (A.n_rows + 31) / 32;
     S.sptr.alloc(size_t(S.n_slices) + 1);
@@ -261,9 +262,10 @@ void copy_sell_bf16(const Sell<double>& S, Sell<float, bf16s>& out, cudaStream_t
     out.n_rows = S.n_rows;
     out.n_cols = S.n_cols;
     out.n_slices = S.n_slices;
-    out.k = S.k;
-    out.r = S.r;
+    out.k = choose_parts(S.nnz, S.n_rows, false);
+    out.r = out.k == 1 ? 1 : 4;
     out.mw = S.mw;
+    out.pw = S.pw;
     out.nnz = S.nnz;
     out.padded = S.padded;
     out.ndiag = 0;
@@ -281,9 +283,10 @@ void copy_sell_f32(const Sell<double>& S, Sell<float>& out, cudaStream_t st)
     out.n_rows = S.n_rows;
     out.n_cols = S.n_cols;
     out.n_slices = S.n_slices;
-    out.k = S.k;
-    out.r = S.r;
+    out.k = choose_parts(S.nnz, S.n_rows, false);
+    out.r = out.k == 1 ? 1 : 4;
     out.mw = S.mw;
+    out.pw = S.pw;
     out.nnz = S.nnz;
     out.padded = S.padded;
     out.ndiag = S.ndiag;

@@ -61,6 +61,7 @@ template <class T, class V = T>
 struct Sell {
     int n_rows = 0, n_cols = 0, n_slices = 0, k = 1, r = 1;
     int mw = 0;        // entries a row of the widest slice
+    int pw = 1;        // warps per row group of the batched kernels: 1 for short rows, 4 for long ones
     int persist = 0;   // 1: row kernels run on a grid of resident blocks that stride over the slices
     int stream = 0;    // coarsest operator only: 1 = its steps stream it through shared memory (coarse_stream.cu)
     int xs = 0;   // coarsest operator only: > 0 = its SpMVs stage x in shared memory, on xs blocks (solve.cu)
@@ -124,22 +125,38 @@ long long mat_bytes32(const Sell<T, V>& s)
     return (s.nnz - s.ndiag) * (long long)(sizeof(V) + 4) + s.ndiag * (long long)sizeof(T);
 }
 
-// Warps per slice from the mean row length: the smallest power of two that
-// leaves at most `per_lane` entries per lane (default 12), capped at
-// `max_parts` (default 8).  Both can be overridden for tuning with
-// AIRG_PER_LANE / AIRG_MAX_PARTS.
-inline int choose_parts(long long nnz, int n_rows)
+// Warps per slice for rows of `avg` entries on average: the smallest power
+// of two that leaves at most `per_lane` entries per lane, capped at
+// `max_parts`.
+inline int parts_for(double avg, int per_lane, int max_parts)
 {
-    static int max_parts = 0, per_lane = 0;
-    if (!max_parts) {
-        const char* e = getenv("AIRG_MAX_PARTS");
-        max_parts = e ? std::max(1, std::min(32, atoi(e))) : 8;
-        const char* q = getenv("AIRG_PER_LANE");
-        per_lane = q ? std::max(1, atoi(q)) : 12;
-    }
-    double avg = n_rows ? double(nnz) / n_rows : 0.0;
     int p = 1;
     while (p < max_parts && avg > double(per_lane) * p) p *= 2;
+    return p;
+}
+
+// Warps per slice of an operator.  At most 12 entries per lane (up to 8
+// warps) give the shortest chains.  In FP64, operators with enough slices to
+// fill the GPU take fewer, because each further warp per slice adds its
+// partial sums to the row (four per warp: with 8, 31 additions on top of a
+// row of 66 products, in the FP64 pipe).  The line, 2800 warps (18 per SM)
+// and at most 48 entries per lane, measured: residual of 70,639 rows of 66
+// entries with 8, 4, 2 warps 32.0, 28.2, 23.6 us; 42,872 rows of 86 with 8,
+// 4, 2: 25.7, 21.1, 25.6 us; smoother term of 117,848 rows of 28 with 4, 2,
+// 1: 23.4, 19.2, 18.1 us; coarse step of 105,946 rows of 67 with 8, 4, 2:
+// 33.5, 29.9, 28.3 us; residual of 17,911 rows of 61 with 8, 4, 2: 13.9,
+// 15.0, 19.9 us.  In FP32, where additions are free, the line gains nothing
+// on average and loses on the longest rows (80,178 of 163: 24.0 -> 27.2 us).
+// AIRG_MAX_PARTS / AIRG_PER_LANE set the cap and the 12, without the line.
+inline int choose_parts(long long nnz, int n_rows, bool fp64)
+{
+    const char* e = getenv("AIRG_MAX_PARTS");
+    const char* q = getenv("AIRG_PER_LANE");
+    const double avg = n_rows ? double(nnz) / n_rows : 0.0;
+    int p = parts_for(avg, q ? std::max(1, atoi(q)) : 12, e ? std::max(1, std::min(32, atoi(e))) : 8);
+    if (e || q || !fp64) return p;
+    const long long slices = (n_rows + 31) / 32;
+    while (p > 1 && avg <= 48.0 * (p / 2) && slices * (p / 2) >= 2800) p /= 2;
     return p;
 }
 
