@@ -159,14 +159,70 @@ __device__ __forceinline__ void xd_win_add(unsigned long long* acc, XdWin& a, do
         : "r"(r0), "r"(r1), "r"(r2), "r"(r3), "r"(r4), "r"(r5), "r"(m));
 }
 
+// Digits lo .. hi of an accumulator, spread too far for the lanes of a warp:
+// one thread walks them.  The accumulator is left altered.
+static __device__ inline double xd_round_serial(unsigned long long* g, int lo, int hi)
+{
+    double r = 0.0;
+    long long* d = reinterpret_cast<long long*>(g);
+    const long long MASK = 0xffffffffLL;
+    long long carry = 0;
+    int top = hi;
+    for (int i = lo; i <= hi; ++i) {
+        const long long v = d[i] + carry;
+        d[i] = v & MASK;
+        carry = v >> 32;                       // floor((v - low) / 2^32)
+    }
+    while (carry != 0 && carry != -1 && top < XD_DIGITS - 1) {
+        d[++top] = carry & MASK;
+        carry >>= 32;
+    }
+    const bool neg = carry < 0;
+    if (neg) {                                 // magnitude: two's complement of the digits
+        long long c = 1;
+        for (int i = lo; i <= top; ++i) {
+            const long long v = (~d[i] & MASK) + c;
+            d[i] = v & MASK;
+            c = v >> 32;
+        }
+        if (c && top < XD_DIGITS - 1) d[++top] = c;
+    }
+    const int last = top;
+    while (top >= lo && d[top] == 0) --top;
+    if (top >= lo) {
+        const int hb = 63 - __clzll(d[top]);
+        const int P = top * 32 + hb;           // most significant bit
+        int lsb = P - 52;                      // last bit kept
+        if (lsb < XD_BIAS - 1074) lsb = XD_BIAS - 1074;
+        auto dig = [&](int i) -> unsigned long long {
+            return i >= lo && i <= last ? (unsigned long long)d[i] : 0ULL;
+        };
+        const int q = lsb >> 5, s = lsb & 31;  // lsb >= XD_BIAS - 1074 > 0
+        unsigned long long M = (dig(q) | (dig(q + 1) << 32)) >> s;
+        if (s) M |= dig(q + 2) << (64 - s);
+        const int rp = lsb - 1;                // rounding bit; the bits below it are sticky
+        const int rb = int((dig(rp >> 5) >> (rp & 31)) & 1ULL);
+        bool sticky = (dig(rp >> 5) & ((1ULL << (rp & 31)) - 1ULL)) != 0ULL;
+        for (int i = lo; i < (rp >> 5) && i <= last && !sticky; ++i) sticky = d[i] != 0;
+        if (rb && (sticky || (M & 1ULL))) M += 1ULL;
+        r = scalbn((double)M, lsb - XD_BIAS);
+        if (neg) r = -r;
+    }
+    return r;
+}
+
 // One warp: carry propagation and round-to-nearest-even of an accumulator in
-// shared memory (which is left altered).  Only the digits between the lowest
-// and the highest nonzero one are walked: the products of one dot product
-// span a few digits of the 140, and the walk is a serial chain.  Every lane
-// gets the result.
+// shared memory.  The products of one dot product touch a few digits of the
+// 140; with at most 28 between the lowest and the highest nonzero one, lane
+// i takes digit lo + i and the whole number, a two's complement of 32 digits,
+// is resolved at once: two local carry steps leave each digit within one unit
+// of its range, and the remaining chains of carries and borrows are a mask
+// addition each (a run of all-ones digits passes a carry on as a run of ones
+// does in an integer).  A thread that walked the digits took about as long as
+// the rest of a small dot product.  Every lane gets the result.
 static __device__ inline double xd_round(unsigned long long* g)
 {
-    const unsigned full = 0xffffffffu;
+    const unsigned full = 0xffffffffu, M = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     int lo = XD_DIGITS, hi = -1;
 #pragma unroll
@@ -178,54 +234,58 @@ static __device__ inline double xd_round(unsigned long long* g)
             hi = k * 32 + 31 - __clz(b);
         }
     }
-    double r = 0.0;
-    if (lane == 0 && hi >= 0) {
-        long long* d = reinterpret_cast<long long*>(g);
-        const long long MASK = 0xffffffffLL;
-        long long carry = 0;
-        int top = hi;
-        for (int i = lo; i <= hi; ++i) {
-            const long long v = d[i] + carry;
-            d[i] = v & MASK;
-            carry = v >> 32;                       // floor((v - low) / 2^32)
-        }
-        while (carry != 0 && carry != -1 && top < XD_DIGITS - 1) {
-            d[++top] = carry & MASK;
-            carry >>= 32;
-        }
-        const bool neg = carry < 0;
-        if (neg) {                                 // magnitude: two's complement of the digits
-            long long c = 1;
-            for (int i = lo; i <= top; ++i) {
-                const long long v = (~d[i] & MASK) + c;
-                d[i] = v & MASK;
-                c = v >> 32;
-            }
-            if (c && top < XD_DIGITS - 1) d[++top] = c;
-        }
-        const int last = top;
-        while (top >= lo && d[top] == 0) --top;
-        if (top >= lo) {
-            const int hb = 63 - __clzll(d[top]);
-            const int P = top * 32 + hb;           // most significant bit
-            int lsb = P - 52;                      // last bit kept
-            if (lsb < XD_BIAS - 1074) lsb = XD_BIAS - 1074;
-            auto dig = [&](int i) -> unsigned long long {
-                return i >= lo && i <= last ? (unsigned long long)d[i] : 0ULL;
-            };
-            const int q = lsb >> 5, s = lsb & 31;  // lsb >= XD_BIAS - 1074 > 0
-            unsigned long long M = (dig(q) | (dig(q + 1) << 32)) >> s;
-            if (s) M |= dig(q + 2) << (64 - s);
-            const int rp = lsb - 1;                // rounding bit; the bits below it are sticky
-            const int rb = int((dig(rp >> 5) >> (rp & 31)) & 1ULL);
-            bool sticky = (dig(rp >> 5) & ((1ULL << (rp & 31)) - 1ULL)) != 0ULL;
-            for (int i = lo; i < (rp >> 5) && i <= last && !sticky; ++i) sticky = d[i] != 0;
-            if (rb && (sticky || (M & 1ULL))) M += 1ULL;
-            r = scalbn((double)M, lsb - XD_BIAS);
-            if (neg) r = -r;
-        }
+    if (hi < 0) return 0.0;
+    if (hi - lo > 27) {
+        const double r = lane == 0 ? xd_round_serial(g, lo, hi) : 0.0;
+        return __shfl_sync(full, r, 0);
     }
-    return __shfl_sync(full, r, 0);
+    // v = l + 2^32 h; each digit passes its h up, twice: t in [-1, 2^32]
+    long long v = lo + lane <= hi ? (long long)g[lo + lane] : 0LL;
+#pragma unroll
+    for (int step = 0; step < 2; ++step) {
+        long long up = __shfl_up_sync(full, v >> 32, 1);
+        if (lane == 0) up = 0;
+        v = (v & 0xffffffffLL) + up;
+    }
+    // digits u = 2^32 generate a carry, all-ones digits pass one on
+    const bool minus = v < 0;                       // -1: a digit 0 that owes one
+    unsigned u = minus ? 0u : unsigned(v);
+    unsigned gen = __ballot_sync(full, v > 0xffffffffLL), pass = __ballot_sync(full, v == 0xffffffffLL);
+    u += (((pass + (gen << 1)) ^ pass) >> lane) & 1u;
+    // then the owed units: digits 0 that owe generate a borrow, digits that
+    // come out 0 pass one on
+    gen = __ballot_sync(full, minus && u == 0u);
+    const unsigned w = u - (minus ? 1u : 0u);
+    pass = __ballot_sync(full, w == 0u);
+    u = w - ((((pass + (gen << 1)) ^ pass) >> lane) & 1u);
+    // magnitude of a negative number (at least four digits above hi hold its sign)
+    const bool neg = __shfl_sync(full, u, 31) >> 31;
+    if (neg) {
+        u = ~u;
+        pass = __ballot_sync(full, u == M);
+        u += (((pass + 1u) ^ pass) >> lane) & 1u;
+    }
+    const unsigned nz = __ballot_sync(full, u != 0u);
+    if (!nz) return 0.0;
+    const int top = 31 - __clz(nz);
+    const int P = (lo + top) * 32 + 31 - __clz(__shfl_sync(full, u, top));   // most significant bit
+    int lsb = P - 52;                               // last bit kept
+    if (lsb < XD_BIAS - 1074) lsb = XD_BIAS - 1074;
+    auto dig = [&](int i) -> unsigned long long {
+        const unsigned x = __shfl_sync(full, u, (i - lo) & 31);
+        return i >= lo && i < lo + 32 ? x : 0u;
+    };
+    const int q = lsb >> 5, s = lsb & 31;           // lsb >= XD_BIAS - 1074 > 0
+    const unsigned long long d0 = dig(q), d1 = dig(q + 1), d2 = dig(q + 2);
+    unsigned long long m = (d0 | (d1 << 32)) >> s;
+    if (s) m |= d2 << (64 - s);
+    const int rp = lsb - 1;                         // rounding bit; the bits below it are sticky
+    const unsigned long long dr = dig(rp >> 5);
+    const bool sticky = (dr & ((1ULL << (rp & 31)) - 1ULL)) != 0ULL ||
+                        __ballot_sync(full, u != 0u && lo + lane < (rp >> 5)) != 0u;
+    if (((dr >> (rp & 31)) & 1ULL) && (sticky || (m & 1ULL))) m += 1ULL;
+    const double r = scalbn((double)m, lsb - XD_BIAS);
+    return neg ? -r : r;
 }
 
 // The products of one block: load(i) reads the operands of element i,
