@@ -618,6 +618,7 @@ struct BatchData {
     HBuf<double> hh;
     struct GEntry { const void* v; void* z; cudaGraphExec_t exec; long long kernels; };
     std::vector<GEntry> graphs;
+    std::vector<std::pair<const void*, void*>> seen;   // pairs used before (graph captured at the second use)
     ~BatchData()
     {
         for (GEntry& g : graphs) cudaGraphExecDestroy(g.exec);
@@ -881,6 +882,10 @@ void bprecond(Hierarchy& H, BatchData& B, const double* v, double* z, cudaStream
     BatchData::GEntry* ge = nullptr;
     for (auto& g : B.graphs)
         if (g.v == v && g.z == z) { ge = &g; break; }
+    if (!ge && first_use(B.seen, v, z)) {
+        bprecond_launch(H, B, v, z, st);
+        return;
+    }
     if (!ge) {
         long long before = S.launches;
         CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
