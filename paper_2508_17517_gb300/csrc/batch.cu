@@ -105,12 +105,13 @@ __device__ __forceinline__ Vals<T, VEC, KW> beach(const F& f, const Vals<T, VEC,
 // time with all their loads issued before their FMAs, which run in entry
 // order.  Then epi(r, L, sums, pre) runs once per row.  `dot` = false skips
 // the product (sums 0).  Every thread of the block reaches the barrier.
-template <class T, int VEC, int KW, int PW, class V, class Pre, class Epi>
-__device__ __forceinline__ void bfor_rows(const SellView<T, V>& S, const T* __restrict__ x, int k, int lg,
+// X: the type x is stored in (FP32 under an FP64 operator: widened exactly).
+template <class T, int VEC, int KW, int PW, class V, class X, class Pre, class Epi>
+__device__ __forceinline__ void bfor_rows(const SellView<T, V>& S, const X* __restrict__ x, int k, int lg,
                                           bool dot, const Pre& pre, const Epi& epi, int rev = 0)
 {
     using LN = Lanes<T, VEC, KW>;
-    using PK = Pack<T, VEC>;
+    using PK = Pack<X, VEC>;
     using PV = decltype(pre(0, LN{}));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int part = warp % PW;
@@ -130,14 +131,20 @@ __device__ __forceinline__ void bfor_rows(const SellView<T, V>& S, const T* __re
     if (valid && dot) {
         if (part == 0 && S.diag) {
             const T dg = __ldg(S.diag + r);
-            acc = beach<T, VEC, KW>([&](T xv) { return dg * xv; }, bload(L, x, r));
+#pragma unroll
+            for (int j = 0; j < KW; ++j)
+                if (L.ok(j)) {
+                    const PK d = *reinterpret_cast<const PK*>(x + size_t(r) * k + L.q(j));
+#pragma unroll
+                    for (int u = 0; u < VEC; ++u) acc.p[j].v[u] = dg * wide<T>(d.v[u]);
+                }
         }
         const int s = r >> 5;
         const int b = S.sptr[s] + (r & 31), w = (S.sptr[s + 1] - S.sptr[s]) >> 5;
         int e = part;
         for (; e + 3 * PW < w; e += 4 * PW) {
             T v[4];
-            const T* xr[4];
+            const X* xr[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int idx = b + 32 * (e + u * PW);
@@ -156,11 +163,11 @@ __device__ __forceinline__ void bfor_rows(const SellView<T, V>& S, const T* __re
                 for (int j = 0; j < KW; ++j)
                     if (L.ok(j))
 #pragma unroll
-                        for (int i = 0; i < VEC; ++i) acc.p[j].v[i] = fma(v[u], xv[u][j].v[i], acc.p[j].v[i]);
+                        for (int i = 0; i < VEC; ++i) acc.p[j].v[i] = fma(v[u], wide<T>(xv[u][j].v[i]), acc.p[j].v[i]);
         }
         if (e < w) {   // up to three entries left, their loads together too
             T v[3];
-            const T* xr[3];
+            const X* xr[3];
             PK xv[3][KW];
 #pragma unroll
             for (int u = 0; u < 3; ++u)
@@ -180,7 +187,7 @@ __device__ __forceinline__ void bfor_rows(const SellView<T, V>& S, const T* __re
                 for (int j = 0; j < KW; ++j)
                     if (e + u * PW < w && L.ok(j))
 #pragma unroll
-                        for (int i = 0; i < VEC; ++i) acc.p[j].v[i] = fma(v[u], xv[u][j].v[i], acc.p[j].v[i]);
+                        for (int i = 0; i < VEC; ++i) acc.p[j].v[i] = fma(v[u], wide<T>(xv[u][j].v[i]), acc.p[j].v[i]);
         }
     }
     if constexpr (PW > 1) {
@@ -214,8 +221,8 @@ struct Vals2 {
     Vals<T, VEC, KW> a, b;
 };
 
-template <class T, int VEC, int KW, int PW>
-__global__ void kb_spmv(SellView<T> S, const T* __restrict__ x, T* __restrict__ y, int k, int lg)
+template <class T, int VEC, int KW, int PW, class X>
+__global__ void kb_spmv(SellView<T> S, const X* __restrict__ x, T* __restrict__ y, int k, int lg)
 {
     using LN = Lanes<T, VEC, KW>;
     using VL = Vals<T, VEC, KW>;
@@ -376,12 +383,6 @@ __global__ void kb_d2f(long long m, const double* a, float* b)
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < m) b[i] = (float)a[i];
 }
-__global__ void kb_f2d(long long m, const float* a, double* b)
-{
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m) b[i] = (double)a[i];
-}
-
 // [q][i] (caller, natural order) <-> [pos(i)][q] (batch, nested order)
 // [q][i] (caller: right-hand sides one after the other, natural order) <->
 // [pos(i)][q] (batch: rows in nested order, right-hand sides adjacent), a
@@ -534,8 +535,8 @@ kb_multiaxpy_norm(long long n, int k, const double* __restrict__ V, long long ld
 }
 
 // x[r][q] += sum_i y[i*k+q] Z_i[r][q] (terms in the order i = 0, 1, ...)
-template <int M>
-__global__ void kb_update(long long n, int k, const double* __restrict__ Zs, long long ldz,
+template <int M, class Z>
+__global__ void kb_update(long long n, int k, const Z* __restrict__ Zs, long long ldz,
                           const double* __restrict__ y, double* __restrict__ x)
 {
     long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -543,18 +544,22 @@ __global__ void kb_update(long long n, int k, const double* __restrict__ Zs, lon
     int q = int(t % k);
     double v[M];
 #pragma unroll
-    for (int i = 0; i < M; ++i) v[i] = __ldg(Zs + i * ldz + t);
+    for (int i = 0; i < M; ++i) v[i] = wide<double>(__ldg(Zs + i * ldz + t));
     double s = x[t];
 #pragma unroll
     for (int i = 0; i < M; ++i) s = fma(y[i * k + q], v[i], s);
     x[t] = s;
 }
 
+// v = w * inv, in FP32 as well where v32 is given (the V-cycle's input)
 __global__ void kb_scale(long long n, int k, const double* __restrict__ w, const double* __restrict__ inv,
-                         double* __restrict__ v)
+                         double* __restrict__ v, float* __restrict__ v32)
 {
     long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n * k) v[t] = w[t] * inv[t % k];
+    if (t >= n * k) return;
+    const double q = w[t] * inv[t % k];
+    v[t] = q;
+    if (v32) v32[t] = float(q);
 }
 
 __global__ void kb_sub(long long m, const double* b, const double* y, double* r)
@@ -611,9 +616,10 @@ BShape bshape(int k)
 struct BatchData {
     int k = 0, m = 0;
     long long nk = 0;
-    DBuf<double> V, Zs, w, bp, xp, r, part, hdev, inv;
+    DBuf<double> V, Zs, w, bp, xp, r, part, hdev, inv;   // Zs: FP64 V-cycle
+    DBuf<float> Zs32;                                    // FP32 V-cycle
     DBuf<double> rwork, t, wa, wb, cr0, cr1, ct, rcs;          // FP64 V-cycle
-    DBuf<float> rwork32, e32, vin32, t32, wa32, wb32, cr032, cr132, ct32, rcs32;  // FP32 V-cycle
+    DBuf<float> rwork32, vin32, t32, wa32, wb32, cr032, cr132, ct32, rcs32;  // FP32 V-cycle
     DBuf<unsigned> ticket;
     HBuf<double> hh;
     struct GEntry { const void* v; void* z; cudaGraphExec_t exec; long long kernels; };
@@ -857,22 +863,21 @@ void bvcycle(SolveData& S, int k, const T* v, T* e, const BWork<T>& wk, cudaStre
     CK_LAUNCH();
 }
 
+// z = M^-1 v: the FP64 V-cycle, or (z an FP32 vector) the FP32 one from
+// vin32, which the kernel that formed the FP64 vector has filled
 void bprecond_launch(Hierarchy& H, BatchData& B, const double* v, double* z, cudaStream_t st)
 {
-    SolveData& S = *H.solve;
-    long long nk = B.nk;
-    if (mixed_precision(H.opt)) {
-        LAUNCH(S, PK_LAYOUT, 12 * nk, kb_d2f<<<grid_for(nk, BT), BT, 0, st>>>(nk, v, B.vin32.p));
-        BWork<float> wk{B.rwork32.p, B.t32.p, B.wa32.p, B.wb32.p, B.cr032.p, B.cr132.p, B.ct32.p, B.rcs32.p};
-        bvcycle<float>(S, B.k, B.vin32.p, B.e32.p, wk, st);
-        LAUNCH(S, PK_LAYOUT, 12 * nk, kb_f2d<<<grid_for(nk, BT), BT, 0, st>>>(nk, B.e32.p, z));
-    } else {
-        BWork<double> wk{B.rwork.p, B.t.p, B.wa.p, B.wb.p, B.cr0.p, B.cr1.p, B.ct.p, B.rcs.p};
-        bvcycle<double>(S, B.k, v, z, wk, st);
-    }
+    BWork<double> wk{B.rwork.p, B.t.p, B.wa.p, B.wb.p, B.cr0.p, B.cr1.p, B.ct.p, B.rcs.p};
+    bvcycle<double>(*H.solve, B.k, v, z, wk, st);
+}
+void bprecond_launch(Hierarchy& H, BatchData& B, const float* v, float* z, cudaStream_t st)
+{
+    BWork<float> wk{B.rwork32.p, B.t32.p, B.wa32.p, B.wb32.p, B.cr032.p, B.cr132.p, B.ct32.p, B.rcs32.p};
+    bvcycle<float>(*H.solve, B.k, v, z, wk, st);
 }
 
-void bprecond(Hierarchy& H, BatchData& B, const double* v, double* z, cudaStream_t st)
+template <class T>
+void bprecond(Hierarchy& H, BatchData& B, const T* v, T* z, cudaStream_t st)
 {
     SolveData& S = *H.solve;
     if (S.prof || !S.use_graphs) {
@@ -925,7 +930,8 @@ void ensure_batch(Hierarchy& H, int k)
     size_t nk = size_t(B->nk);
     int m = B->m;
     B->V.alloc(size_t(m + 1) * nk);
-    B->Zs.alloc(size_t(m) * nk);
+    if (mixed_precision(H.opt)) B->Zs32.alloc(size_t(m) * nk);
+    else B->Zs.alloc(size_t(m) * nk);
     B->w.alloc(nk); B->bp.alloc(nk); B->xp.alloc(nk); B->r.alloc(nk);
     B->part.alloc(size_t(RG) * (MAXB + 1) * k);
     B->hdev.alloc(size_t(3 * (MAXB + 2)) * k);
@@ -936,7 +942,7 @@ void ensure_batch(Hierarchy& H, int k)
     size_t nf = size_t(std::max({S.max_nf, S.max_nc, 1})) * k, nc = size_t(std::max(S.n_coarse, 1)) * k;
     const size_t nrc = S.smooth_type != AIRG_SMOOTH_F ? size_t(std::max<long long>(S.rc_total, 1)) * k : 0;
     if (mixed_precision(H.opt)) {
-        B->rwork32.alloc(nk); B->e32.alloc(nk); B->vin32.alloc(nk);
+        B->rwork32.alloc(nk); B->vin32.alloc(nk);
         B->t32.alloc(nf); B->wa32.alloc(nf); B->wb32.alloc(nf);
         B->cr032.alloc(nc); B->cr132.alloc(nc); B->ct32.alloc(nc);
         if (nrc) B->rcs32.alloc(nrc);
@@ -976,6 +982,9 @@ void solve_batched(Hierarchy& H, int k, const double* b, double* x, double rtol,
     const int g = grid_for(nk, BT);
     SellView<double> A = view(S.Atop);
     const long long topB = mat_bytes32(S.Atop) + 16 * nk;
+    const bool mixed = mixed_precision(H.opt);
+    float* v32 = mixed ? B.vin32.p : nullptr;
+    const long long scaleB = (mixed ? 20 : 16) * nk;
     LAUNCH(S, PK_LAYOUT, 20 * nk, kb_to_nested<<<grid_tiles(n, k), 256, 0, st>>>(n, k, S.pos0.p, b, B.bp.p));
     LAUNCH(S, PK_LAYOUT, 20 * nk, kb_to_nested<<<grid_tiles(n, k), 256, 0, st>>>(n, k, S.pos0.p, x, B.xp.p));
     std::vector<double> bn, rn, tol(k);
@@ -983,7 +992,7 @@ void solve_batched(Hierarchy& H, int k, const double* b, double* x, double rtol,
     for (int q = 0; q < k; ++q) tol[q] = std::max(rtol * bn[q], atol);
     auto residual = [&]() {
         LAUNCH_F(S, PK_TOPSPMV, topB, 2 * S.Atop.nnz * k,
-               WITH_BATCH(double, k, S.Atop, kb_spmv<double, VEC, KW, PW><<<grid_rows(n, PW, lg), BT, 0, st>>>(A, B.xp.p, B.w.p, k, lg)));
+               WITH_BATCH(double, k, S.Atop, kb_spmv<double, VEC, KW, PW, double><<<grid_rows(n, PW, lg), BT, 0, st>>>(A, B.xp.p, B.w.p, k, lg)));
         LAUNCH_F(S, PK_KRYLOV, 24 * nk, nk, kb_sub<<<g, BT, 0, st>>>(nk, B.bp.p, B.w.p, B.r.p));
         bnorms(S, B, B.r.p, rn, st);
     };
@@ -999,9 +1008,15 @@ void solve_batched(Hierarchy& H, int k, const double* b, double* x, double rtol,
                 nact += rn[q] > tol[q];
             }
             if (!nact) break;
-            bprecond(H, B, B.r.p, B.Zs.p, st);
             h2d(B.hdev.p, yq.data(), size_t(k), st);
-            LAUNCH_F(S, PK_KRYLOV, 24 * nk, 2 * nk, kb_update<1><<<g, BT, 0, st>>>(n, k, B.Zs.p, nk, B.hdev.p, B.xp.p));
+            if (mixed) {
+                LAUNCH(S, PK_LAYOUT, 12 * nk, kb_d2f<<<g, BT, 0, st>>>(nk, B.r.p, B.vin32.p));
+                bprecond(H, B, (const float*)B.vin32.p, B.Zs32.p, st);
+                LAUNCH_F(S, PK_KRYLOV, 20 * nk, 2 * nk, kb_update<1, float><<<g, BT, 0, st>>>(n, k, B.Zs32.p, nk, B.hdev.p, B.xp.p));
+            } else {
+                bprecond(H, B, (const double*)B.r.p, B.Zs.p, st);
+                LAUNCH_F(S, PK_KRYLOV, 24 * nk, 2 * nk, kb_update<1, double><<<g, BT, 0, st>>>(n, k, B.Zs.p, nk, B.hdev.p, B.xp.p));
+            }
             residual();
             ++its;
         }
@@ -1023,13 +1038,20 @@ void solve_batched(Hierarchy& H, int k, const double* b, double* x, double rtol,
         std::fill(gv.begin(), gv.end(), 0.0);
         for (int q = 0; q < k; ++q) gv[q] = rn[q];
         h2d(B.inv.p, inv.data(), size_t(k), st);
-        LAUNCH_F(S, PK_KRYLOV, 16 * nk, nk, kb_scale<<<g, BT, 0, st>>>(n, k, B.r.p, B.inv.p, B.V.p));
+        LAUNCH_F(S, PK_KRYLOV, scaleB, nk, kb_scale<<<g, BT, 0, st>>>(n, k, B.r.p, B.inv.p, B.V.p, v32));
         for (int j = 0; j < m; ++j) {
             double* vj = B.V.p + size_t(j) * nk;
-            double* zj = B.Zs.p + size_t(j) * nk;
-            bprecond(H, B, vj, zj, st);
-            LAUNCH_F(S, PK_TOPSPMV, topB, 2 * S.Atop.nnz * k,
-                   WITH_BATCH(double, k, S.Atop, kb_spmv<double, VEC, KW, PW><<<grid_rows(n, PW, lg), BT, 0, st>>>(A, zj, B.w.p, k, lg)));
+            if (mixed) {
+                float* zj = B.Zs32.p + size_t(j) * nk;
+                bprecond(H, B, (const float*)B.vin32.p, zj, st);
+                LAUNCH_F(S, PK_TOPSPMV, topB - 4 * nk, 2 * S.Atop.nnz * k,
+                       WITH_BATCH(double, k, S.Atop, kb_spmv<double, VEC, KW, PW, float><<<grid_rows(n, PW, lg), BT, 0, st>>>(A, zj, B.w.p, k, lg)));
+            } else {
+                double* zj = B.Zs.p + size_t(j) * nk;
+                bprecond(H, B, (const double*)vj, zj, st);
+                LAUNCH_F(S, PK_TOPSPMV, topB, 2 * S.Atop.nnz * k,
+                       WITH_BATCH(double, k, S.Atop, kb_spmv<double, VEC, KW, PW, double><<<grid_rows(n, PW, lg), BT, 0, st>>>(A, zj, B.w.p, k, lg)));
+            }
             // CGS with a second pass only if the first cancelled, for some
             // active right-hand side, more than reorth_ratio() allows
             double* h1 = B.hdev.p;
@@ -1091,8 +1113,8 @@ void solve_batched(Hierarchy& H, int k, const double* b, double* x, double rtol,
             }
             if (!still || its >= maxit || j + 1 == m) break;
             h2d(B.inv.p, inv.data(), size_t(k), st);
-            LAUNCH_F(S, PK_KRYLOV, 16 * nk, nk,
-                   kb_scale<<<g, BT, 0, st>>>(n, k, B.w.p, B.inv.p, B.V.p + size_t(j + 1) * nk));
+            LAUNCH_F(S, PK_KRYLOV, scaleB, nk,
+                   kb_scale<<<g, BT, 0, st>>>(n, k, B.w.p, B.inv.p, B.V.p + size_t(j + 1) * nk, v32));
         }
         // least squares per right-hand side, zero-padded to the common width
         int jmax = 0;
@@ -1108,8 +1130,12 @@ void solve_batched(Hierarchy& H, int k, const double* b, double* x, double rtol,
         }
         if (jmax) {
             h2d(B.hdev.p, Y.data(), size_t(jmax) * k, st);
-            LAUNCH_F(S, PK_KRYLOV, 8LL * nk * (jmax + 2), 2LL * nk * jmax,
-                   WITH_M(jmax, kb_update<MM><<<g, BT, 0, st>>>(n, k, B.Zs.p, nk, B.hdev.p, B.xp.p)));
+            if (mixed)
+                LAUNCH_F(S, PK_KRYLOV, 4LL * nk * (jmax + 4), 2LL * nk * jmax,
+                       WITH_M(jmax, kb_update<MM, float><<<g, BT, 0, st>>>(n, k, B.Zs32.p, nk, B.hdev.p, B.xp.p)));
+            else
+                LAUNCH_F(S, PK_KRYLOV, 8LL * nk * (jmax + 2), 2LL * nk * jmax,
+                       WITH_M(jmax, kb_update<MM, double><<<g, BT, 0, st>>>(n, k, B.Zs.p, nk, B.hdev.p, B.xp.p)));
         }
         residual();
     }

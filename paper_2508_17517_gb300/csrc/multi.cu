@@ -164,7 +164,7 @@ cudaGraphExec_t capture_richardson(airg_batch_s& B)
             CK(cudaStreamWaitEvent(st, B.fork, 0));
             airg::mp_vcycle(H, S.r.p, S.Zs.p, st);
             airg::mp_add_dev(H, S.Zs.p, B.act[p].p, S.xp.p, st);
-            airg::mp_residual(H, S.bp.p, S.xp.p, S.w.p, S.r.p, st);
+            airg::mp_residual(H, S.bp.p, S.xp.p, S.r.p, st);
             airg::mp_multidot(H, 0, S.V.p, S.r.p, dv + o.rn(), 1, st);
             CK(cudaEventRecord(B.join[p], st));
             CK(cudaStreamWaitEvent(B.master, B.join[p], 0));
@@ -304,7 +304,7 @@ void solve_multi(airg_batch_s& B, const double* const* b, double* const* x, bool
         airg::mp_permute(H, bd, S.bp.p, true, B.ps[p]);
         airg::mp_permute(H, xd, S.xp.p, true, B.ps[p]);
         airg::mp_multidot(H, 0, S.V.p, S.bp.p, B.dv[p].p + o.bn(), 1, B.ps[p]);
-        airg::mp_residual(H, S.bp.p, S.xp.p, S.w.p, S.r.p, B.ps[p]);
+        airg::mp_residual(H, S.bp.p, S.xp.p, S.r.p, B.ps[p]);
         airg::mp_multidot(H, 0, S.V.p, S.r.p, B.dv[p].p + o.rn(), 1, B.ps[p]);
         st[p].Hm.assign(size_t(m + 1) * m, 0.0);
         st[p].cs.assign(m, 0.0);
@@ -447,7 +447,7 @@ void solve_multi(airg_batch_s& B, const double* const* b, double* const* x, bool
                 airg::h2d(B.dv[p].p + o.y(), s.y.data(), size_t(jd), B.ps[p]);
                 airg::mp_update(H, jd, S.Zs.p, B.dv[p].p + o.y(), S.xp.p, B.ps[p]);
             }
-            airg::mp_residual(H, S.bp.p, S.xp.p, S.w.p, S.r.p, B.ps[p]);
+            airg::mp_residual(H, S.bp.p, S.xp.p, S.r.p, B.ps[p]);
             airg::mp_multidot(H, 0, S.V.p, S.r.p, B.dv[p].p + o.rn(), 1, B.ps[p]);
         }
         sync_all(B);
@@ -501,6 +501,7 @@ airg_status airg_setup_batch(int nprob, const airg_csr* As, const airg_options* 
         for (int p = 0; p < nprob; ++p) {
             airg::DevCSR D = airg::upload_csr_checked(&As[p], st);
             B->H.push_back(airg::build_hierarchy(std::move(D), o, st));
+            airg::prepare_multi(*B->H.back());
         }
         B->m = B->H[0]->solve->restart;
         Off of{B->m};

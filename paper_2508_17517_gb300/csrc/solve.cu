@@ -239,7 +239,7 @@ __global__ void k_d2f(long long n, const double* a, float* b)
 __global__ void k_f2d(long long n, const float* a, double* b)
 {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) b[i] = (double)a[i];
+    if (i < n) b[i] = widen(a[i]);
 }
 
 // FP64 value -> FP32 (round to nearest) -> bfloat16, rounding the 16
@@ -364,9 +364,11 @@ __device__ __forceinline__ int ldcol(const int* __restrict__ col, const unsigned
 }
 
 // C16: column indices from the 16-bit copy, cb + col16 (the same values)
-template <class T, int U = 4, class V = T, bool C16 = false>
+// X: the type x is stored in (FP32 where an FP64 operator reads the FP32
+// V-cycle's result; widened exactly)
+template <class T, int U = 4, class V = T, bool C16 = false, class X>
 __device__ __forceinline__ T strided_dot(const int* __restrict__ col, const unsigned short* __restrict__ col16,
-                                         int cb, const V* __restrict__ val, const T* __restrict__ x, int idx,
+                                         int cb, const V* __restrict__ val, const X* __restrict__ x, int idx,
                                          int end, int stride)
 {
     static_assert(U % 4 == 0, "U must be a multiple of 4");
@@ -380,7 +382,7 @@ __device__ __forceinline__ T strided_dot(const int* __restrict__ col, const unsi
             v[u] = ldval<T>(val + idx + u * stride);
         }
 #pragma unroll
-        for (int u = 0; u < U; ++u) xv[u] = x[c[u]];
+        for (int u = 0; u < U; ++u) xv[u] = wide<T>(x[c[u]]);
 #pragma unroll
         for (int u = 0; u < U; ++u) a[u % 4] = fma(v[u], xv[u], a[u % 4]);
     }
@@ -394,7 +396,7 @@ __device__ __forceinline__ T strided_dot(const int* __restrict__ col, const unsi
             v[u] = ok ? ldval<T>(val + idx + u * stride) : T(0);
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) xv[u] = idx + u * stride < end ? x[c[u]] : T(0);
+        for (int u = 0; u < 4; ++u) xv[u] = idx + u * stride < end ? wide<T>(x[c[u]]) : T(0);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
             if (idx + u * stride < end) a[u] = fma(v[u], xv[u], a[u]);
@@ -406,9 +408,9 @@ __device__ __forceinline__ T strided_dot(const int* __restrict__ col, const unsi
 // that share the slice (part = this warp's index among them).  Every thread
 // of the block must call it (it synchronises the block when P > 1).  The
 // sum is valid in the part-0 warp, which also adds the dense diagonal.
-template <class T, int P, int U = 4, class V = T, bool C16 = false>
+template <class T, int P, int U = 4, class V = T, bool C16 = false, class X>
 __device__ __forceinline__ T row_dot(const SellView<T, V>& S, int slice, int lane, int part,
-                                     const T* __restrict__ x)
+                                     const X* __restrict__ x)
 {
     T acc = T(0);
     if (slice < S.n_slices) {
@@ -429,14 +431,14 @@ __device__ __forceinline__ T row_dot(const SellView<T, V>& S, int slice, int lan
         __syncthreads();
     }
     const int r = slice * 32 + lane;
-    if (S.diag && part == 0 && r < S.n_rows) acc = fma(S.diag[r], x[r], acc);
+    if (S.diag && part == 0 && r < S.n_rows) acc = fma(S.diag[r], wide<T>(x[r]), acc);
     return acc;
 }
 
 // G slices of at most MW entries a row each: all loads of the G rows of a
 // lane, then all gathers, then the sums.
-template <class T, int G, int MW, class V, bool C16>
-__device__ __forceinline__ void dot_narrow(const SellView<T, V>& S, const T* __restrict__ x, const int* b,
+template <class T, int G, int MW, class V, bool C16, class X>
+__device__ __forceinline__ void dot_narrow(const SellView<T, V>& S, const X* __restrict__ x, const int* b,
                                            const int* w, const int* cb, T* acc)
 {
     int c[G][MW];
@@ -452,7 +454,7 @@ __device__ __forceinline__ void dot_narrow(const SellView<T, V>& S, const T* __r
 #pragma unroll
     for (int q = 0; q < G; ++q)
 #pragma unroll
-        for (int u = 0; u < MW; ++u) xv[q][u] = u < w[q] ? x[c[q][u]] : T(0);
+        for (int u = 0; u < MW; ++u) xv[q][u] = u < w[q] ? wide<T>(x[c[q][u]]) : T(0);
 #pragma unroll
     for (int q = 0; q < G; ++q)
 #pragma unroll
@@ -475,8 +477,8 @@ __device__ __forceinline__ void dot_narrow(const SellView<T, V>& S, const T* __r
 // term of level 0 (7.3M rows, MW = 1) 92 -> 52 us FP64, 47 -> 32 us FP32;
 // residual of level 0 (MW = 2) 100 -> 84 us FP64; restriction of levels 3 and
 // 4 (8 to 16 slots, MW = 0) 88 -> 76 and 70 -> 62 us FP64.
-template <class T, int R, class V, bool C16, int MW>
-__device__ __forceinline__ void dot_slices(const SellView<T, V>& S, const T* __restrict__ x, int s0, int lane,
+template <class T, int R, class V, bool C16, int MW, class X>
+__device__ __forceinline__ void dot_slices(const SellView<T, V>& S, const X* __restrict__ x, int s0, int lane,
                                            T (&acc)[R])
 {
     int b[R], w[R], cb[R];
@@ -491,7 +493,7 @@ __device__ __forceinline__ void dot_slices(const SellView<T, V>& S, const T* __r
         w[q] = (p1 - p0) >> 5;
         fits = fits && w[q] <= 4;
         const int r = s * 32 + lane;
-        acc[q] = (S.diag && r < S.n_rows) ? __ldg(S.diag + r) * x[r] : T(0);
+        acc[q] = (S.diag && r < S.n_rows) ? __ldg(S.diag + r) * wide<T>(x[r]) : T(0);
     }
     if constexpr (MW == 1 || MW == 2) {
         dot_narrow<T, R, MW, V, C16>(S, x, b, w, cb, acc);
@@ -514,7 +516,7 @@ __device__ __forceinline__ void dot_slices(const SellView<T, V>& S, const T* __r
                 v[u] = ok ? ldval<T>(S.val + b[q] + 32 * (u0 + u)) : T(0);
             }
 #pragma unroll
-            for (int u = 0; u < U; ++u) xv[u] = u0 + u < w[q] ? x[c[u]] : T(0);
+            for (int u = 0; u < U; ++u) xv[u] = u0 + u < w[q] ? wide<T>(x[c[u]]) : T(0);
 #pragma unroll
             for (int u = 0; u < U; ++u)
                 if (u0 + u < w[q]) acc[q] = fma(v[u], xv[u], acc[q]);
@@ -528,8 +530,8 @@ __device__ __forceinline__ void dot_slices(const SellView<T, V>& S, const T* __r
 // slice wider than one, two entries), 1 (four on average) or 0 (more).  R = slices per warp for K = 1, and
 // loads in flight per lane (4, 8 or 16) for K > 1; in neither case does R
 // change the arithmetic.
-template <class T, int K, int R, bool C16 = false, class V, class Pre, class Epi>
-__device__ __forceinline__ void for_rows(const SellView<T, V>& S, const T* __restrict__ x, const Pre& pre,
+template <class T, int K, int R, bool C16 = false, class V, class X, class Pre, class Epi>
+__device__ __forceinline__ void for_rows(const SellView<T, V>& S, const X* __restrict__ x, const Pre& pre,
                                          const Epi& epi, int rev = 0)
 {
     using PV = decltype(pre(0));
@@ -580,10 +582,23 @@ struct Pair {
 };
 
 // y = S x
-template <class T, int K, int R, class V = T, bool C16 = false>
-__global__ void k_spmv(SellView<T, V> S, const T* __restrict__ x, T* __restrict__ y)
+template <class T, int K, int R, class V = T, bool C16 = false, class X = T>
+__global__ void k_spmv(SellView<T, V> S, const X* __restrict__ x, T* __restrict__ y)
 {
     for_rows<T, K, R, C16>(S, x, [](int) { return 0; }, [&](int r, T d, int) { y[r] = d; });
+}
+
+// r = b - S x, in FP32 as well where r32 is given (the V-cycle's input)
+template <int K, int R, bool C16 = false>
+__global__ void k_residual(SellView<double> S, const double* __restrict__ x, const double* __restrict__ b,
+                           double* __restrict__ res, float* __restrict__ r32)
+{
+    for_rows<double, K, R, C16>(S, x, [&](int r) { return b[r]; },
+                                [&](int r, double d, double br) {
+                                    const double q = br - d;
+                                    res[r] = q;
+                                    if (r32) r32[r] = float(q);
+                                });
 }
 
 // restriction (R = [Z I] of Eq. 4): dst_c[k] = src_c[k] + (Z src_f)[k]; the
@@ -1065,7 +1080,7 @@ __device__ __forceinline__ T row_dot_rt(const SellView<T>& S, int slice, int lan
     T acc = T(0);
     if (slice < S.n_slices) {
         int b = S.sptr[slice], w = (S.sptr[slice + 1] - b) >> 5;
-        acc = strided_dot(S.col, S.col16, 0, S.val, x, b + lane + 32 * part, b + lane + 32 * w, 32 * P);
+        acc = strided_dot<T>(S.col, S.col16, 0, S.val, x, b + lane + 32 * part, b + lane + 32 * w, 32 * P);
     }
     if (P > 1) {
         const int warp = threadIdx.x >> 5;
@@ -1199,12 +1214,12 @@ k_multidot(long long n, const double* __restrict__ V, long long ldv, const doubl
     if (threadIdx.x == 0) *ticket = 0u;
 }
 
-// w += sum_i c_i V_i with c_i = -h_i (neg) or h_i, the terms added in the
-// order i = 0, 1, ...; with norm, *out = ||w||^2 of the result (partial sums
+// w += sum_i c_i V_i (V stored as Z, FP32 widened exactly) with c_i = -h_i
+// (neg) or h_i, the terms added in the order i = 0, 1, ...; with norm, *out = ||w||^2 of the result (partial sums
 // per block, fixed-order sum in the last block).
-template <int M>
+template <int M, class Z>
 __global__ void __launch_bounds__(RB)
-k_multiaxpy(long long n, const double* __restrict__ V, long long ldv, const double* __restrict__ h, int neg,
+k_multiaxpy(long long n, const Z* __restrict__ V, long long ldv, const double* __restrict__ h, int neg,
             double* __restrict__ w, int norm, double* __restrict__ part, double* __restrict__ out,
             unsigned* ticket)
 {
@@ -1217,7 +1232,7 @@ k_multiaxpy(long long n, const double* __restrict__ V, long long ldv, const doub
     for (long long r = (long long)blockIdx.x * RB + threadIdx.x; r < n; r += (long long)gridDim.x * RB) {
         double v[M];
 #pragma unroll
-        for (int u = 0; u < M; ++u) v[u] = __ldg(V + u * ldv + r);
+        for (int u = 0; u < M; ++u) v[u] = wide<double>(__ldg(V + u * ldv + r));
         double s = w[r];
 #pragma unroll
         for (int u = 0; u < M; ++u) s = fma(c[u], v[u], s);
@@ -1253,26 +1268,25 @@ k_multiaxpy(long long n, const double* __restrict__ V, long long ldv, const doub
 }
 
 
-__global__ void k_scale_into(long long n, const double* __restrict__ w, double inv, double* __restrict__ v)
+// v = w * inv, in FP32 as well where v32 is given (the V-cycle's input)
+__global__ void k_scale_into(long long n, const double* __restrict__ w, double inv, double* __restrict__ v,
+                             float* __restrict__ v32)
 {
     long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < n) v[r] = w[r] * inv;
+    if (r >= n) return;
+    const double q = w[r] * inv;
+    v[r] = q;
+    if (v32) v32[r] = float(q);
 }
 
-// r = b - y
-// x += z, unless *active is 0 (a frozen problem of a batch)
-__global__ void k_add_dev(long long n, const double* __restrict__ z, const int* __restrict__ active,
+// x += z (stored as Z), unless *active is 0 (a frozen problem of a batch)
+template <class Z>
+__global__ void k_add_dev(long long n, const Z* __restrict__ z, const int* __restrict__ active,
                           double* __restrict__ x)
 {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || (active && !*active)) return;
-    x[i] += z[i];
-}
-
-__global__ void k_sub2(long long n, const double* b, const double* y, double* r)
-{
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) r[i] = b[i] - y[i];
+    x[i] += wide<double>(z[i]);
 }
 
 // nested <-> natural permutation
@@ -2092,14 +2106,15 @@ void build_solve_data(Hierarchy& H, cudaStream_t st)
         else S->rcs.alloc(nrc);
     }
     if (mixed_precision(H.opt)) {
-        S->rwork32.alloc(n0); S->e32.alloc(n0); S->vin32.alloc(n0);
+        S->rwork32.alloc(n0); S->vin32.alloc(n0);
         S->t32.alloc(nf); S->wa32.alloc(nf); S->wb32.alloc(nf);
         S->cr032.alloc(nc); S->cr132.alloc(nc); S->ct32.alloc(nc);
     }
     S->restart = std::max(1, H.opt.gmres_restart);
     int m = S->restart;
     S->V.alloc(size_t(m + 1) * n0);
-    S->Zs.alloc(size_t(m) * n0);
+    if (mixed_precision(H.opt)) S->Zs32.alloc(size_t(m) * n0);
+    else S->Zs.alloc(size_t(m) * n0);
     S->w.alloc(n0); S->bp.alloc(n0); S->xp.alloc(n0); S->r.alloc(n0);
     S->part.alloc(size_t(RGRID) * (m + 2));
     S->hdev.alloc(size_t(3 * (m + 2)));
@@ -2134,14 +2149,15 @@ void launch_multidot(SolveData& S, long long n, int m, const double* V, long lon
 
 // w += sum_i (neg ? -h_i : h_i) V_i (chunks of MCH); nrm2 (if not null)
 // receives ||w||^2 of the result
-void launch_multiaxpy(SolveData& S, long long n, int m, const double* V, long long ldv, const double* h,
+template <class Z>
+void launch_multiaxpy(SolveData& S, long long n, int m, const Z* V, long long ldv, const double* h,
                       int neg, double* w, double* nrm2, cudaStream_t st)
 {
     for (int c0 = 0; c0 < m; c0 += MCH) {
         const int mc = std::min(MCH, m - c0);
         const int norm = nrm2 && c0 + mc == m;
-        LAUNCH_F(S, PK_KRYLOV, 8LL * n * (mc + 2), 2LL * n * (mc + (norm ? 1 : 0)),
-               WITH_M(mc, k_multiaxpy<MM><<<RGRID, RB, 0, st>>>(n, V + c0 * ldv, ldv, h + c0, neg, w, norm,
+        LAUNCH_F(S, PK_KRYLOV, (long long)sizeof(Z) * n * mc + 16LL * n, 2LL * n * (mc + (norm ? 1 : 0)),
+               WITH_M(mc, k_multiaxpy<MM, Z><<<RGRID, RB, 0, st>>>(n, V + c0 * ldv, ldv, h + c0, neg, w, norm,
                                                                  S.part.p, nrm2, S.ticket.p)));
     }
 }
@@ -2171,63 +2187,56 @@ void precond_launch(Hierarchy& H, const double* v, double* z, cudaStream_t st)
     }
 }
 
-// z = M^-1 v: replays the captured V-cycle graph of this (v, z) pair.  The
-// first time a pair is used its kernels are launched directly: capturing and
-// instantiating a graph of 50 to 130 kernels costs 0.3 to 0.6 ms, which a
-// hierarchy that solves once never gets back.
-void precond(Hierarchy& H, const double* v, double* z, cudaStream_t st)
+// Captures `launch` (kernels on st) into an executable graph.
+template <class F>
+cudaGraphExec_t capture(cudaStream_t st, const F& launch)
 {
-    SolveData& S = *H.solve;
+    CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+    try {
+        launch();
+    } catch (...) {
+        cudaGraph_t g0;
+        cudaStreamEndCapture(st, &g0);
+        if (g0) cudaGraphDestroy(g0);
+        throw;
+    }
+    cudaGraph_t graph;
+    CK(cudaStreamEndCapture(st, &graph));
+    cudaGraphExec_t exec;
+    cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
+    cudaGraphDestroy(graph);
+    CK(e);
+    return exec;
+}
+
+// Runs the V-cycle `launch` from v to z: replays the captured graph of this
+// (v, z) pair.  The first time a pair is used its kernels are launched
+// directly: capturing and instantiating a graph of 50 to 130 kernels costs
+// 0.3 to 0.6 ms, which a hierarchy that solves once never gets back.
+template <class F>
+void replay(SolveData& S, const void* v, void* z, cudaStream_t st, const F& launch)
+{
     if (!S.use_graphs) {
-        precond_launch(H, v, z, st);
+        launch();
         return;
     }
     if (S.prof) {
         // profiled V-cycle: captured afresh with its event pairs, so that the
         // kernels run as in an unprofiled solve (no host launch gaps)
-        CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        try {
-            precond_launch(H, v, z, st);
-        } catch (...) {
-            cudaGraph_t g0;
-            cudaStreamEndCapture(st, &g0);
-            if (g0) cudaGraphDestroy(g0);
-            throw;
-        }
-        cudaGraph_t graph;
-        CK(cudaStreamEndCapture(st, &graph));
-        cudaGraphExec_t exec;
-        cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
-        cudaGraphDestroy(graph);
-        CK(e);
-        S.prof_execs.push_back(exec);
-        CK(cudaGraphLaunch(exec, st));
+        S.prof_execs.push_back(capture(st, launch));
+        CK(cudaGraphLaunch(S.prof_execs.back(), st));
         return;
     }
     SolveData::GEntry* ge = nullptr;
     for (auto& g : S.graphs)
         if (g.v == v && g.z == z) { ge = &g; break; }
     if (!ge && first_use(S.seen, v, z)) {
-        precond_launch(H, v, z, st);
+        launch();
         return;
     }
     if (!ge) {
         long long before = S.launches;
-        CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        try {
-            precond_launch(H, v, z, st);
-        } catch (...) {
-            cudaGraph_t g0;
-            cudaStreamEndCapture(st, &g0);
-            if (g0) cudaGraphDestroy(g0);
-            throw;
-        }
-        cudaGraph_t graph;
-        CK(cudaStreamEndCapture(st, &graph));
-        cudaGraphExec_t exec;
-        cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
-        cudaGraphDestroy(graph);
-        CK(e);
+        cudaGraphExec_t exec = capture(st, launch);
         long long nk = S.launches - before;
         S.launches = before;
         S.graphs.push_back(SolveData::GEntry{v, z, exec, nk});
@@ -2235,6 +2244,22 @@ void precond(Hierarchy& H, const double* v, double* z, cudaStream_t st)
     }
     CK(cudaGraphLaunch(ge->exec, st));
     S.launches += ge->kernels;
+}
+
+// z = M^-1 v with the FP64 V-cycle
+void precond(Hierarchy& H, const double* v, double* z, cudaStream_t st)
+{
+    replay(*H.solve, v, z, st, [&] { precond_launch(H, v, z, st); });
+}
+
+// The FP32 V-cycle from vin32, which the kernel that formed the FP64 vector
+// has filled, straight into z: the outer iteration keeps its preconditioned
+// vectors in FP32, which is all they hold, and reads them from there.
+void precond_mixed(Hierarchy& H, float* z, cudaStream_t st)
+{
+    SolveData& S = *H.solve;
+    VWork<float> wk{S.rwork32.p, S.t32.p, S.wa32.p, S.wb32.p, nullptr, S.cr032.p, S.cr132.p, S.ct32.p, S.rcs32.p};
+    replay(S, S.vin32.p, z, st, [&] { vcycle<float>(S, S.vin32.p, z, wk, st); });
 }
 
 void richardson(Hierarchy& H, double rtol, double atol, int maxit, airg_solve_info& info,
@@ -2253,27 +2278,36 @@ void fgmres(Hierarchy& H, double rtol, double atol, int maxit, airg_solve_info& 
     double bn = dev_norm(S, S.bp.p, n, st);
     double tol = std::max(rtol * bn, atol);
     int its = 0;
+    const bool mixed = mixed_precision(H.opt);
     auto residual = [&]() {
-        LAUNCH_F(S, PK_TOPSPMV, topB, 2 * S.Atop.nnz,
-               WITH_KR_COL(S.Atop, k_spmv<double, KK, RR, double, C16><<<grid_rows(S.Atop, k_spmv<double, KK, RR, double, C16>), block_rows(S.Atop), 0, st>>>(A, S.xp.p, S.w.p)));
-        LAUNCH_F(S, PK_KRYLOV, 24 * n, n, k_sub2<<<g, TB, 0, st>>>(n, S.bp.p, S.w.p, S.r.p));
+        LAUNCH_F(S, PK_TOPSPMV, topB + 8 * n, 2 * S.Atop.nnz + n,
+               WITH_KR_COL(S.Atop, k_residual<KK, RR, C16><<<grid_rows(S.Atop, k_residual<KK, RR, C16>), block_rows(S.Atop), 0, st>>>(A, S.xp.p, S.bp.p, S.r.p, nullptr)));
         CK_LAUNCH();
         return dev_norm(S, S.r.p, n, st);
     };
     double rn = residual();
     std::vector<double> Hm(size_t(m + 1) * m), cs(m), sn(m), gv(m + 1), y(m);
     double* hh = S.hhost.p;
+    float* v32 = mixed ? S.vin32.p : nullptr;
+    const long long scaleB = (mixed ? 20 : 16) * n;
     while (rn > tol && its < maxit) {
-        LAUNCH_F(S, PK_KRYLOV, 16 * n, n, k_scale_into<<<g, TB, 0, st>>>(n, S.r.p, 1.0 / rn, S.V.p));
+        LAUNCH_F(S, PK_KRYLOV, scaleB, n, k_scale_into<<<g, TB, 0, st>>>(n, S.r.p, 1.0 / rn, S.V.p, v32));
         std::fill(gv.begin(), gv.end(), 0.0);
         gv[0] = rn;
         int jdone = 0;
         for (int j = 0; j < m; ++j) {
             double* vj = S.V.p + size_t(j) * n;
-            double* zj = S.Zs.p + size_t(j) * n;
-            precond(H, vj, zj, st);
-            LAUNCH_F(S, PK_TOPSPMV, topB, 2 * S.Atop.nnz,
-                   WITH_KR_COL(S.Atop, k_spmv<double, KK, RR, double, C16><<<grid_rows(S.Atop, k_spmv<double, KK, RR, double, C16>), block_rows(S.Atop), 0, st>>>(A, zj, S.w.p)));
+            if (mixed) {
+                float* zj = S.Zs32.p + size_t(j) * n;
+                precond_mixed(H, zj, st);
+                LAUNCH_F(S, PK_TOPSPMV, topB - 4 * n, 2 * S.Atop.nnz,
+                       WITH_KR_COL(S.Atop, k_spmv<double, KK, RR, double, C16, float><<<grid_rows(S.Atop, k_spmv<double, KK, RR, double, C16, float>), block_rows(S.Atop), 0, st>>>(A, zj, S.w.p)));
+            } else {
+                double* zj = S.Zs.p + size_t(j) * n;
+                precond(H, vj, zj, st);
+                LAUNCH_F(S, PK_TOPSPMV, topB, 2 * S.Atop.nnz,
+                       WITH_KR_COL(S.Atop, k_spmv<double, KK, RR, double, C16><<<grid_rows(S.Atop, k_spmv<double, KK, RR, double, C16>), block_rows(S.Atop), 0, st>>>(A, zj, S.w.p)));
+            }
             // classical Gram-Schmidt; a second pass only when the first
             // one cancelled enough of ||w|| to cost orthogonality:
             // ||w'||^2 < reorth_ratio() ||w||^2
@@ -2315,8 +2349,8 @@ void fgmres(Hierarchy& H, double rtol, double atol, int maxit, airg_solve_info& 
             ++its;
             jdone = j + 1;
             if (std::fabs(gv[j + 1]) <= tol || its >= maxit || den == 0.0 || hn == 0.0) break;
-            LAUNCH_F(S, PK_KRYLOV, 16 * n, n,
-                   k_scale_into<<<g, TB, 0, st>>>(n, S.w.p, 1.0 / hn, S.V.p + size_t(j + 1) * n));
+            LAUNCH_F(S, PK_KRYLOV, scaleB, n,
+                   k_scale_into<<<g, TB, 0, st>>>(n, S.w.p, 1.0 / hn, S.V.p + size_t(j + 1) * n, v32));
         }
         for (int j = jdone - 1; j >= 0; --j) {
             double s = gv[j];
@@ -2324,7 +2358,8 @@ void fgmres(Hierarchy& H, double rtol, double atol, int maxit, airg_solve_info& 
             y[j] = s / Hm[size_t(j) * m + j];
         }
         h2d(S.hdev.p, y.data(), jdone, st);
-        launch_multiaxpy(S, n, jdone, S.Zs.p, n, S.hdev.p, 0, S.xp.p, nullptr, st);
+        if (mixed) launch_multiaxpy(S, n, jdone, S.Zs32.p, n, S.hdev.p, 0, S.xp.p, nullptr, st);
+        else launch_multiaxpy(S, n, jdone, S.Zs.p, n, S.hdev.p, 0, S.xp.p, nullptr, st);
         CK_LAUNCH();
         rn = residual();
     }
@@ -2346,18 +2381,23 @@ void richardson(Hierarchy& H, double rtol, double atol, int maxit, airg_solve_in
     const long long topB = mat_bytes(S.Atop) + 16 * n;
     double bn = dev_norm(S, S.bp.p, n, st);
     double tol = std::max(rtol * bn, atol);
+    const bool mixed = mixed_precision(H.opt);
     auto residual = [&]() {
-        LAUNCH_F(S, PK_TOPSPMV, topB, 2 * S.Atop.nnz,
-               WITH_KR_COL(S.Atop, k_spmv<double, KK, RR, double, C16><<<grid_rows(S.Atop, k_spmv<double, KK, RR, double, C16>), block_rows(S.Atop), 0, st>>>(A, S.xp.p, S.w.p)));
-        LAUNCH_F(S, PK_KRYLOV, 24 * n, n, k_sub2<<<g, TB, 0, st>>>(n, S.bp.p, S.w.p, S.r.p));
+        LAUNCH_F(S, PK_TOPSPMV, topB + 8 * n, 2 * S.Atop.nnz + n,
+               WITH_KR_COL(S.Atop, k_residual<KK, RR, C16><<<grid_rows(S.Atop, k_residual<KK, RR, C16>), block_rows(S.Atop), 0, st>>>(A, S.xp.p, S.bp.p, S.r.p, mixed ? S.vin32.p : nullptr)));
         CK_LAUNCH();
         return dev_norm(S, S.r.p, n, st);
     };
     double rn = residual();
     int its = 0;
     while (rn > tol && its < maxit) {
-        precond(H, S.r.p, S.Zs.p, st);
-        LAUNCH_F(S, PK_KRYLOV, 24 * n, n, k_add_dev<<<g, TB, 0, st>>>(n, S.Zs.p, nullptr, S.xp.p));
+        if (mixed) {
+            precond_mixed(H, S.Zs32.p, st);
+            LAUNCH_F(S, PK_KRYLOV, 20 * n, n, k_add_dev<<<g, TB, 0, st>>>(n, (const float*)S.Zs32.p, nullptr, S.xp.p));
+        } else {
+            precond(H, S.r.p, S.Zs.p, st);
+            LAUNCH_F(S, PK_KRYLOV, 24 * n, n, k_add_dev<<<g, TB, 0, st>>>(n, (const double*)S.Zs.p, nullptr, S.xp.p));
+        }
         rn = residual();
         ++its;
     }
@@ -2415,12 +2455,25 @@ void mp_scale_dev(Hierarchy& H, const double* w, const double* nrm2, const int* 
     LAUNCH_F(S, PK_KRYLOV, 16 * n, n, k_scale_dev<<<grid_for(n, TB), TB, 0, st>>>(n, w, nrm2, active, v));
 }
 
-void mp_residual(Hierarchy& H, const double* b, const double* x, double* y, double* r, cudaStream_t st)
+void mp_residual(Hierarchy& H, const double* b, const double* x, double* r, cudaStream_t st)
 {
     SolveData& S = *H.solve;
     long long n = S.n0;
-    mp_top_spmv(H, x, y, st);
-    LAUNCH_F(S, PK_KRYLOV, 24 * n, n, k_sub2<<<grid_for(n, TB), TB, 0, st>>>(n, b, y, r));
+    SellView<double> A = view(S.Atop);
+    LAUNCH_F(S, PK_TOPSPMV, mat_bytes(S.Atop) + 24 * n, 2 * S.Atop.nnz + n,
+           WITH_KR_COL(S.Atop, k_residual<KK, RR, C16><<<grid_rows(S.Atop, k_residual<KK, RR, C16>), block_rows(S.Atop), 0, st>>>(A, x, b, r, nullptr)));
+}
+
+// Buffers of the many-grid forms, which keep every vector of the outer
+// iteration in FP64: the single solve's FP32 ones give way.
+void prepare_multi(Hierarchy& H)
+{
+    SolveData& S = *H.solve;
+    if (!mixed_precision(H.opt)) return;
+    const size_t n = size_t(std::max(S.n0, 1));
+    S.Zs32.release();
+    S.Zs.alloc(size_t(S.restart) * n);
+    S.e32.alloc(n);
 }
 
 void mp_update(Hierarchy& H, int m, const double* Zs, const double* y, double* x, cudaStream_t st)

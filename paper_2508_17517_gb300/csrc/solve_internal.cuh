@@ -93,6 +93,25 @@ SellView<T, V> view(const Sell<T, V>& s)
                           s.col16.n ? s.col16.p : nullptr, s.cbase.n ? s.cbase.p : nullptr};
 }
 
+// FP32 -> FP64, exactly.  The conversion instruction runs at the rate of the
+// FP64 pipe (2 per clock and SM), which the kernels that widen are short of;
+// normal numbers and zeros are widened with integer operations.
+__device__ __forceinline__ double widen(float f)
+{
+    const unsigned u = __float_as_uint(f), m = u & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)            // normal
+        return __hiloint2double(int((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), int(u << 29));
+    if (m == 0u) return __hiloint2double(int(u), 0);
+    return double(f);                             // subnormal, inf, nan
+}
+// a vector element in the arithmetic type
+template <class T, class X>
+__device__ __forceinline__ T wide(X x)
+{
+    if constexpr (sizeof(T) == 8 && sizeof(X) == 4) return widen(x);
+    else return x;
+}
+
 // stored value -> arithmetic type
 template <class T, class V>
 __device__ __forceinline__ T ldval(const V* p)
@@ -222,7 +241,8 @@ struct SolveData {
     DBuf<float> rcs32;
     // outer FGMRES
     int restart = 0;
-    DBuf<double> V, Zs, w, bp, xp, r, part;
+    DBuf<double> V, Zs, w, bp, xp, r, part;   // Zs: FP64 V-cycle, and the many-grid forms
+    DBuf<float> Zs32;            // preconditioned vectors of the FP32 V-cycle
     DBuf<double> hdev;
     HBuf<double> hhost;
     long long bytes_vcycle = 0;
@@ -422,7 +442,8 @@ void mp_multiaxpy_norm(Hierarchy& H, int m, const double* V, const double* h, do
                        cudaStream_t st);
 void mp_scale_dev(Hierarchy& H, const double* w, const double* nrm2, const int* active, double* v,
                   cudaStream_t st);
-void mp_residual(Hierarchy& H, const double* b, const double* x, double* y, double* r, cudaStream_t st);
+void mp_residual(Hierarchy& H, const double* b, const double* x, double* r, cudaStream_t st);
+void prepare_multi(Hierarchy& H);
 void mp_update(Hierarchy& H, int m, const double* Zs, const double* y, double* x, cudaStream_t st);
 void mp_permute(Hierarchy& H, const double* a, double* b, bool to_nested, cudaStream_t st);
 void mp_add_dev(Hierarchy& H, const double* z, const int* active, double* x, cudaStream_t st);
