@@ -95,7 +95,9 @@ SellView<T, V> view(const Sell<T, V>& s)
 
 // FP32 -> FP64, exactly.  The conversion instruction runs at the rate of the
 // FP64 pipe (2 per clock and SM), which the kernels that widen are short of;
-// normal numbers and zeros are widened with integer operations.
+// normal numbers and zeros are widened with integer operations (32
+// right-hand sides on 2048^2, FP32 preconditioned vectors: 161.5 ms with the
+// conversion, 148.5 with this; FP64 vectors: 157.0).
 __device__ __forceinline__ double widen(float f)
 {
     const unsigned u = __float_as_uint(f), m = u & 0x7fffffffu;
