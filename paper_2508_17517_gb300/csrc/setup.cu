@@ -22,6 +22,7 @@
 #include "exact_dot.cuh"
 #include "handle.h"
 #include "hostmath.h"
+#include "setup_index.h"
 
 namespace airg {
 
@@ -913,13 +914,13 @@ __global__ void k_gemm_pack(int m, const int* __restrict__ toff, const int* __re
 // Rows of the overflow list: tables in global memory, one warp each.  The
 // entries of A's row are taken one at a time, in column order, by the whole
 // warp; the lanes share that entry's row of B, whose columns are distinct.
-__global__ void k_gemm_table_size(int nlist, const int* list, const int* prod, int* tsize)
+// tsize: slots of each row's table, -1 for more than 32-bit offsets reach.
+__global__ void k_gemm_table_size(int nlist, const int* list, const int* prod, int n_cols, int* tsize)
 {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nlist) return;
-    int sz = 1;
-    while (sz < 2 * prod[list[t]]) sz <<= 1;
-    tsize[t] = sz;
+    const long long size = gemm_table_slots(prod[list[t]], n_cols);
+    tsize[t] = size <= GEMM_MAX_SLOTS ? int(size) : -1;
 }
 
 __global__ void k_gemm_hash_global(int nlist, const int* list, int row0, const int* arp, const int* aci,
@@ -1445,10 +1446,12 @@ void gemm_piece(const DevCSR& A, const DevCSR& B, const int* prod, const int* ro
     const int nover = nc[3] ? read1(counts.p + 4, st) : 0;
     if (nover) {
         DBuf<int> tsize(static_cast<size_t>(nover));
-        k_gemm_table_size<<<grid_for(nover, TB), TB, 0, st>>>(nover, over.p, prod, tsize.p);
+        k_gemm_table_size<<<grid_for(nover, TB), TB, 0, st>>>(nover, over.p, prod, B.n_cols, tsize.p);
         CK_LAUNCH();
         std::vector<int> ts(static_cast<size_t>(nover));
         d2h(ts.data(), tsize.p, size_t(nover), st);
+        for (int t : ts)
+            if (t < 0) fail(AIRG_ERR_OOM, "a row of a sparse product may have more than 2^29 columns");
         for (int t0 = 0; t0 < nover;) {
             Run R;
             R.first = t0;
@@ -1505,7 +1508,7 @@ void spgemm(const DevCSR& A, const DevCSR& B, DevCSR& C, cudaStream_t st)
     static long long kLimit = 0;
     if (!kLimit) {
         const char* e = getenv("AIRG_SPGEMM_SLOTS");   // tuning / testing override
-        kLimit = e ? std::max(1LL, atoll(e)) : (1LL << 28);
+        kLimit = gemm_piece_limit(e ? atoll(e) : (1LL << 28));
     }
     DBuf<int> prod(size_t(std::max(m, 1))), room(size_t(std::max(m, 1)));
     DBuf<unsigned long long> sum(1);
