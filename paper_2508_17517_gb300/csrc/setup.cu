@@ -509,7 +509,7 @@ __global__ void k_fsp_power_warp(int n, const int* rp, const int* ci, const doub
                                  const double* tprev, double* tout)
 {
     const int lane = threadIdx.x & 31;
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long i = warp_index(blockIdx.x, blockDim.x, threadIdx.x);
     if (i >= n) return;
     const int r0 = rp[i], r1 = rp[i + 1];
     if (r1 - r0 < FSP_WARP_ROW) return;
@@ -637,7 +637,7 @@ __global__ void k_gemm_lanes(int nlist, const int* __restrict__ list, int row0, 
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, g = lane & (G - 1);
-    const int at = (blockIdx.x * blockDim.x + threadIdx.x) / G;
+    const long long at = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const bool row = at < nlist;                  // uniform over the group
     if (!__any_sync(full, row)) return;
     const int li = row ? list[at] : 0, i = row0 + li;
@@ -1074,7 +1074,8 @@ __global__ void k_drop_rows_warp(int n, const int* __restrict__ rp, const double
                                  int8_t* __restrict__ keep, int* __restrict__ cnt)
 {
     const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31, i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    const long long i = warp_index(blockIdx.x, blockDim.x, threadIdx.x);
     if (i >= n) return;
     const int b = rp[i], e = rp[i + 1];
     double m = 0.0;
@@ -1098,7 +1099,8 @@ __global__ void k_drop_lump_warp(int n, const int* __restrict__ rp, const int* _
                                  double* __restrict__ vout, int* __restrict__ cnt, int* bad)
 {
     const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31, i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    const long long i = warp_index(blockIdx.x, blockDim.x, threadIdx.x);
     if (i >= n) return;
     const int b = rp[i], e = rp[i + 1];
     double m = 0.0;
@@ -1144,7 +1146,8 @@ __global__ void k_compact_warp(int n, const int* __restrict__ rp, const int* __r
                                const int* __restrict__ nrp, int* __restrict__ nci, double* __restrict__ nv)
 {
     const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31, i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    const long long i = warp_index(blockIdx.x, blockDim.x, threadIdx.x);
     if (i >= n) return;
     const int b = rp[i], e = rp[i + 1];
     int o = nrp[i];

@@ -1,4 +1,4 @@
-// Sizes of the setup's sparse products, on the host and on the device.
+// Sizes and indexes of the setup's kernels, on the host and on the device.
 #pragma once
 
 #ifdef __CUDACC__
@@ -8,6 +8,13 @@
 #endif
 
 namespace airg {
+
+// The warp of a launch that a thread belongs to.  In 64 bits: one warp per
+// row passes 2^32 threads at 2^27 rows, a size that the setup accepts.
+AIRG_HD inline long long warp_index(unsigned block, unsigned block_threads, unsigned thread)
+{
+    return ((long long)block * block_threads + thread) >> 5;
+}
 
 constexpr long long GEMM_MAX_SLOTS = 1LL << 30;   // table offsets are 32-bit
 

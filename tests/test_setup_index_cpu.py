@@ -42,3 +42,10 @@ def test_sparse_product_table_sizes(tmp_path):
                   "gemm_table_slots((1LL << 29) + 1, 2147483647) <= GEMM_MAX_SLOTS",
                   "gemm_piece_limit(-5)", "gemm_piece_limit(4096)", "gemm_piece_limit(1LL << 40)") == \
         [1, 0, 1, 4096, 2**30]
+
+
+def test_warp_per_row_index(tmp_path):
+    """Row of a thread where one warp takes a row, up to 2^31 rows: with
+    blocks of 256 threads the thread number passes 2^32 at row 2^27."""
+    rows = [0, 7, 8, 2**27 - 1, 2**27, 2**27 + 9, 2**31 - 1]
+    assert values(tmp_path, *["warp_index(%du, 256u, %du)" % (r // 8, r % 8 * 32 + 31) for r in rows]) == rows
