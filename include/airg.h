@@ -422,9 +422,10 @@ airg_status airg_operator_layout_info(const airg_handle* h, int level, int op, a
 /*
  * Failure-detection check of the device-side waits: launches one block that
  * waits, through the same bounded wait as the grid barrier of the
- * persistent kernels, for an arrival that never comes.  The wait must give
- * up after `spin_limit` polls of ~50 ns, record the error flag and let the
- * kernel finish; the call then returns AIRG_ERR_TIMEOUT (the designed
+ * persistent kernels, for an arrival that never comes, and then one that
+ * waits so through the bounded wait of the setup's Gram-Schmidt columns.
+ * Each must give up after `spin_limit` polls, record the error flag and let
+ * the kernel finish; the call then returns AIRG_ERR_TIMEOUT (the designed
  * outcome) and the CUDA context stays usable.  Any other status means the
  * mechanism is broken.  Nothing hangs or faults.
  */

@@ -520,7 +520,8 @@ airg_status airg_check_wait_timeout(int64_t spin_limit, void* stream)
     bool gave_up = false;
     airg_status st = guarded([&] {
         if (spin_limit < 1) airg::fail(AIRG_ERR_ARG, "spin_limit must be positive");
-        gave_up = airg::barrier_timeout_check(spin_limit, (cudaStream_t)stream);
+        gave_up = airg::barrier_timeout_check(spin_limit, (cudaStream_t)stream) &&
+                  airg::column_timeout_check(spin_limit, (cudaStream_t)stream);
         if (!gave_up) airg::fail(AIRG_ERR_STATE, "the bounded wait did not report its timeout");
     });
     if (st == AIRG_OK && gave_up) {

@@ -434,6 +434,35 @@ k_mgs_xdot(long long n, double* __restrict__ w, const double* __restrict__ vprev
     if (xd_grid_sum(sacc, gacc, ticket)) xd_write(sacc[0], bad, out, out_sqrt);
 }
 
+constexpr int XC_WARPS = 16, XC_THREADS = XC_WARPS * 32, XC_MAX_E = 8;
+constexpr long long XC_SPIN_LIMIT = 2000000;   // ~1 s of polls
+
+// One thread: waits until *arrivals has reached target; false, with *err
+// set, after `limit` polls without it or once *err is set.
+__device__ __forceinline__ bool xc_wait(unsigned* arrivals, unsigned target, int* err, long long limit)
+{
+    for (long long spins = 0;; ++spins) {
+        unsigned seen;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(arrivals) : "memory");
+        if (int(seen - target) >= 0) return true;
+        if (spins >= limit) {
+            atomicExch(err, 1);
+            return false;
+        }
+        if ((spins & 1023) == 1023 && *(volatile int*)err) return false;
+    }
+}
+
+// Failure-detection check: one block waits for a second one's arrival, which
+// never comes, and must give up after `limit` polls.
+// state: [arrivals, err], zero.
+static __global__ void k_column_timeout_check(unsigned* state, long long limit)
+{
+    if (threadIdx.x != 0) return;
+    atomicAdd(state, 1u);
+    xc_wait(state, 2u, reinterpret_cast<int*>(state + 1), limit);
+}
+
 // One column of a modified Gram-Schmidt process in one launch: for i = 0..j
 // h_i = <w, v_i> (correctly rounded), w <- w - (h_i v_i) (product rounded,
 // then the difference), then h_{j+1} = ||w|| and v_{j+1} = w / h_{j+1}.  The
@@ -450,20 +479,23 @@ k_mgs_xdot(long long n, double* __restrict__ w, const double* __restrict__ vprev
 // summed there by earlier launches, mod 3; the accumulator two places ahead
 // is cleared behind each barrier, before the next one.
 //   arrivals: counter of barrier arrivals, `base` of them by earlier
-// launches.  err: set when the bounded wait gives up (the launch then runs
-// to its end).  One block needs none of these.
-constexpr int XC_WARPS = 16, XC_THREADS = XC_WARPS * 32, XC_MAX_E = 8;
-constexpr long long XC_SPIN_LIMIT = 2000000;   // ~1 s of polls
-
+// launches.  One block needs none of these.
+//   The wait for the other blocks is bounded.  A block that gives up (`limit`
+// polls, or another block's word that it did) sets *err and ends there, so
+// nothing is ever computed from an incomplete sum: w and the earlier columns
+// are as they were, hcol, vnext and the accumulators are not to be used, and
+// the caller takes the column from w again, one launch per dot.
 template <int E>
 static __global__ void __launch_bounds__(XC_THREADS, 1)
 k_mgs_column(int n, const double* __restrict__ V, int j, const double* __restrict__ w,
              double* __restrict__ vnext, double* __restrict__ hcol, unsigned long long* gdig, int phase,
-             unsigned* arrivals, unsigned base, int* bad, int* err)
+             unsigned* arrivals, unsigned base, int* bad, int* err, long long limit)
 {
     __shared__ unsigned long long sacc[XC_WARPS][XD_DIGITS];
     __shared__ unsigned long long tot[XD_DIGITS];
     __shared__ double hs;
+    __shared__ bool gave_up;
+    if (threadIdx.x == 0) gave_up = false;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int t = threadIdx.x; t < XC_WARPS * XD_DIGITS; t += XC_THREADS) (&sacc[0][0])[t] = 0ULL;
     const int i0 = blockIdx.x * (XC_THREADS * E) + threadIdx.x;
@@ -506,17 +538,7 @@ k_mgs_column(int n, const double* __restrict__ V, int j, const double* __restric
             if (gridDim.x > 1) {
                 if (lane == 0) {
                     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrivals) : "memory");
-                    const unsigned target = base + gridDim.x * unsigned(i + 1);
-                    unsigned seen;
-                    for (long long spins = 0;; ++spins) {
-                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(arrivals) : "memory");
-                        if (int(seen - target) >= 0) break;
-                        if ((spins & 1023) == 1023 && *(volatile int*)err) break;
-                        if (spins > XC_SPIN_LIMIT) {
-                            atomicExch(err, 1);
-                            break;
-                        }
-                    }
+                    gave_up = !xc_wait(arrivals, base + gridDim.x * unsigned(i + 1), err, limit);
                 }
                 __syncwarp();
                 for (int t = lane; t < XD_DIGITS; t += 32) tot[t] = __ldcg(g + t);
@@ -535,6 +557,7 @@ k_mgs_column(int n, const double* __restrict__ V, int j, const double* __restric
             }
         }
         __syncthreads();
+        if (gave_up) return;
         const double h = hs;
         if (i > j) {
 #pragma unroll

@@ -65,6 +65,7 @@ std::unique_ptr<Hierarchy> build_hierarchy(DevCSR&& A0, const airg_options& opt,
                                            cudaStream_t st);
 void dot_exact_device(long long n, const double* x, const double* y, double* out,
                       double* out_sqrt, cudaStream_t st);
+bool column_timeout_check(long long limit, cudaStream_t st);
 void rng_uniform_device(uint64_t seed, long long level, long long purpose, long long n,
                         double* out, cudaStream_t st);
 void csr_transpose(const DevCSR& A, DevCSR& T, cudaStream_t st);

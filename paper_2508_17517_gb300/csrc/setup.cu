@@ -1267,12 +1267,14 @@ struct Ctx {
     DBuf<unsigned> xticket;          // last-block ticket of k_xdot
     long long ndots = 0;             // exact dot products launched
     HBuf<double> hcol;               // one Hessenberg column on the host
-    // grid state of k_mgs_column: accumulators, [arrivals, error], and what
+    // grid state of k_mgs_column: accumulators, barrier arrivals, and what
     // earlier launches left there
     DBuf<unsigned long long> cdig;
     DBuf<unsigned> cbar;
     unsigned cbase = 0;
     int cphase = 0;
+    bool columns = true;             // false once a launch of it gave up waiting
+    long long spin_limit = XC_SPIN_LIMIT;
     explicit Ctx(cudaStream_t s) : st(s)
     {
         xacc.alloc(XD_DIGITS);
@@ -1282,9 +1284,10 @@ struct Ctx {
         CK(cudaMemsetAsync(xbad.p, 0, xbad.bytes(), st));
         CK(cudaMemsetAsync(xticket.p, 0, xticket.bytes(), st));
         cdig.alloc(3 * XD_DIGITS);
-        cbar.alloc(2);
+        cbar.alloc(1);
         CK(cudaMemsetAsync(cdig.p, 0, cdig.bytes(), st));
         CK(cudaMemsetAsync(cbar.p, 0, cbar.bytes(), st));
+        if (const char* e = getenv("AIRG_COLUMN_SPINS")) spin_limit = std::max(0LL, atoll(e));
     }
 };
 
@@ -1320,11 +1323,14 @@ void mgs_xdot(Ctx& c, long long n, double* w, const double* vprev, const double*
 }
 
 // Column j of the Gram-Schmidt process of w (length n) against v_0 .. v_j,
-// one launch; false where a row's worth of registers per SM does not hold w.
+// one launch; false where a row's worth of registers per SM does not hold w,
+// where the blocks cannot be resident together (a GPU shared out by SMs), or
+// after a launch that gave up waiting.  *err is set by one that does.
 // Few elements a thread as long as blocks are left: a block's share of the
 // integer work is ~0.25 us per element and thread, another block adds little
 // to the barrier; up to 2048 elements one block has no barrier at all.
-bool mgs_column(Ctx& c, long long n, const double* V, int j, const double* w, double* vnext, double* hcol)
+bool mgs_column(Ctx& c, long long n, const double* V, int j, const double* w, double* vnext, double* hcol,
+                int* err)
 {
     const long long per = XC_THREADS, sms = num_sms();
     int E = 1;
@@ -1334,7 +1340,7 @@ bool mgs_column(Ctx& c, long long n, const double* V, int j, const double* w, do
         while (E < XC_MAX_E && (n + per * E - 1) / (per * E) > sms) E *= 2;
         grid = (n + per * E - 1) / (per * E);
     }
-    if (grid > sms || grid < 1) return false;
+    if (!c.columns || grid > sms || grid < 1) return false;
     auto launch = [&](auto kernel) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(unsigned(grid));
@@ -1345,13 +1351,19 @@ bool mgs_column(Ctx& c, long long n, const double* V, int j, const double* w, do
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = grid > 1 ? 1 : 0;
-        CK(cudaLaunchKernelEx(&cfg, kernel, int(n), V, j, w, vnext, hcol, c.cdig.p, c.cphase, c.cbar.p, c.cbase,
-                              c.xbad.p, reinterpret_cast<int*>(c.cbar.p + 1)));
+        return cudaLaunchKernelEx(&cfg, kernel, int(n), V, j, w, vnext, hcol, c.cdig.p, c.cphase, c.cbar.p, c.cbase,
+                                  c.xbad.p, err, c.spin_limit);
     };
-    if (E == 1) launch(k_mgs_column<1>);
-    else if (E == 2) launch(k_mgs_column<2>);
-    else if (E == 4) launch(k_mgs_column<4>);
-    else launch(k_mgs_column<8>);
+    const cudaError_t e = E == 1   ? launch(k_mgs_column<1>)
+                          : E == 2 ? launch(k_mgs_column<2>)
+                          : E == 4 ? launch(k_mgs_column<4>)
+                                   : launch(k_mgs_column<8>);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        (void)cudaGetLastError();
+        c.columns = false;
+        return false;
+    }
+    CK(e);
     c.ndots += j + 2;
     if (grid > 1) {
         c.cbase += unsigned(grid) * unsigned(j + 2);
@@ -1619,9 +1631,12 @@ ArnoldiOut arnoldi(Ctx& c, const DevCSR& A, const double* b, int m, double tol, 
 {
     cudaStream_t st = c.st;
     long long n = A.n_rows;
-    // H on the device by columns, so that one copy brings a column to the host
-    DBuf<double> V(size_t(m + 1) * n), w(n), Hd(size_t(m + 1) * m + 1);
-    double* beta_d = Hd.p + size_t(m + 1) * m;
+    // H on the device by columns, each behind the word that its launch sets
+    // when it gives up, so that one copy brings both to the host
+    const size_t ld = size_t(m) + 2;
+    DBuf<double> V(size_t(m + 1) * n), w(n), Hd(ld * m + 1);
+    CK(cudaMemsetAsync(Hd.p, 0, Hd.bytes(), st));
+    double* beta_d = Hd.p + ld * m;
     xdot(c, n, b, b, nullptr, beta_d);
     int g = grid_for(n, TB);
     k_div_dev<<<g, TB, 0, st>>>(n, V.p, b, beta_d);
@@ -1630,24 +1645,31 @@ ArnoldiOut arnoldi(Ctx& c, const DevCSR& A, const double* b, int m, double tol, 
     const double beta_h = read1(beta_d, st);
     ArnoldiOut out;
     out.k = m;
-    c.hcol.alloc(size_t(m) + 1);
-    const double* col = c.hcol.p;
+    c.hcol.alloc(ld);
+    const double* col = c.hcol.p + 1;
     for (int j = 0; j < m; ++j) {
         k_spmv_det<<<grid_for(n, TB), TB, 0, st>>>(int(n), A.rp.p, A.ci.p, A.v.p, V.p + size_t(j) * n, w.p);
         CK_LAUNCH();
         // h_ij = <w, v_i> then w -= h_ij v_i, for i = 0..j (modified
         // Gram-Schmidt), and v_{j+1} = w / ||w||: in one launch where w fits
-        // in registers, else one per dot (each update fused with the next)
-        double* hj = Hd.p + size_t(j) * (m + 1);
+        // in registers, else, or where that launch gave up, one per dot (each
+        // update fused with the next)
+        double* hj = Hd.p + ld * j + 1;
         double* hn = hj + j + 1;
-        const bool column = mgs_column(c, n, V.p, j, w.p, V.p + size_t(j + 1) * n, hj);
-        if (!column) {
+        auto dots = [&] {
             for (int i = 0; i <= j; ++i)
                 mgs_xdot(c, n, w.p, i ? V.p + size_t(i - 1) * n : nullptr, i ? hj + i - 1 : nullptr,
                          V.p + size_t(i) * n, hj + i, nullptr);
             mgs_xdot(c, n, w.p, V.p + size_t(j) * n, hj + j, nullptr, nullptr, hn);
+        };
+        bool column = mgs_column(c, n, V.p, j, w.p, V.p + size_t(j + 1) * n, hj, reinterpret_cast<int*>(hj - 1));
+        if (!column) dots();
+        d2h(c.hcol.p, hj - 1, size_t(j) + 3, st);
+        if (*reinterpret_cast<const int*>(c.hcol.p)) {
+            c.columns = column = false;
+            dots();
+            d2h(c.hcol.p + 1, hj, size_t(j) + 2, st);
         }
-        d2h(c.hcol.p, hj, size_t(j) + 2, st);
         for (int i = 0; i <= j + 1; ++i) Hh[size_t(i) * m + j] = col[i];
         double s = 0.0;
         for (int i = 0; i <= j + 1; ++i) s = s + col[i] * col[i];
@@ -1672,7 +1694,6 @@ ArnoldiOut arnoldi(Ctx& c, const DevCSR& A, const double* b, int m, double tol, 
             CK_LAUNCH();
         }
     }
-    if (read1(c.cbar.p + 1, st)) fail(AIRG_ERR_TIMEOUT, "a grid barrier of the Gram-Schmidt kernel gave up waiting");
     out.beta = beta_h;
     int k = out.k;
     out.H.assign(size_t(k + 1) * k, 0.0);
@@ -1936,6 +1957,17 @@ void cf_split(Ctx& c, SetupLevel& L, const airg_options& o, int level)
 }  // namespace
 
 // ===========================================================================
+// Runs the bounded wait of k_mgs_column for an arrival that never comes;
+// true if it gave up, as designed.
+bool column_timeout_check(long long limit, cudaStream_t st)
+{
+    DBuf<unsigned> state(2);
+    CK(cudaMemsetAsync(state.p, 0, state.bytes(), st));
+    k_column_timeout_check<<<1, 32, 0, st>>>(state.p, limit);
+    CK_LAUNCH();
+    return read1(state.p + 1, st) != 0;
+}
+
 void dot_exact_device(long long n, const double* x, const double* y, double* out,
                       double* out_sqrt, cudaStream_t st)
 {
