@@ -964,22 +964,93 @@ __global__ void k_gemm_hash_global(int nlist, const int* list, int row0, const i
     if (lane == 0) cnt[list[at]] = run_cnt[at] = c;
 }
 
-// Their entries in column order, packed: an entry's rank is the number of
-// smaller columns in its table.
-__global__ void k_gemm_emit_global(const int* toff, const int* keys, const double* vals, const int* crp, int* cci,
-                                   double* cv)
+// Their entries in column order, packed, one block per row: the table's
+// occupied slots go to the row's place, are sorted by column EMIT_CHUNK at a
+// time in shared memory, and in rows of several chunks each entry's rank is
+// its position in its own chunk plus its lower bounds in the others (the
+// columns of a row are distinct).  The sorted chunks wait in the table, which
+// has at least twice as many slots as the row has entries and is not needed
+// any more.  Bound: latency of the scan of the table, which is read once.
+// Ranking every entry against all slots, of a table sized by the products,
+// took entries x slots reads: setup of 3,142 rows of 61 entries (coarse rows
+// of 2,048) 1160 -> 18.8 ms, of 6,354 rows 4067 -> 46.4 ms.
+constexpr int EMIT_CHUNK = 2048;
+
+__global__ void __launch_bounds__(TB)
+k_gemm_emit_global(const int* toff, int* keys, double* vals, const int* crp, int* cci, double* cv)
 {
-    const int o = crp[blockIdx.x], t0 = toff[blockIdx.x], t1 = toff[blockIdx.x + 1];
-    for (int t = t0 + threadIdx.x; t < t1; t += blockDim.x) {
-        const int key = keys[t];
-        if (key < 0) continue;
-        int r = 0;
-        for (int q = t0; q < t1; ++q) {
-            const int k = keys[q];
-            r += k >= 0 && k < key;
+    __shared__ int k[EMIT_CHUNK];
+    __shared__ double v[EMIT_CHUNK];
+    __shared__ int filled;
+    const int lane = threadIdx.x & 31;
+    const int o = crp[blockIdx.x], n = crp[blockIdx.x + 1] - o, t0 = toff[blockIdx.x], t1 = toff[blockIdx.x + 1];
+    if (threadIdx.x == 0) filled = 0;
+    __syncthreads();
+    for (int tb = t0; tb < t1; tb += TB) {
+        const int t = tb + threadIdx.x;
+        const int key = t < t1 ? keys[t] : -1;
+        const unsigned b = __ballot_sync(0xffffffffu, key >= 0);
+        int at = 0;
+        if (lane == 0 && b) at = atomicAdd(&filled, __popc(b));
+        at = o + __shfl_sync(0xffffffffu, at, 0) + __popc(b & ((1u << lane) - 1u));
+        if (key >= 0) {
+            cci[at] = key;
+            cv[at] = vals[t];
+        }
+    }
+    __syncthreads();
+    for (int c0 = 0; c0 < n; c0 += EMIT_CHUNK) {
+        const int m = min(EMIT_CHUNK, n - c0);
+        int size = 1;
+        while (size < m) size <<= 1;
+        for (int t = threadIdx.x; t < size; t += TB) {
+            k[t] = t < m ? cci[o + c0 + t] : 0x7fffffff;
+            v[t] = t < m ? cv[o + c0 + t] : 0.0;
+        }
+        __syncthreads();
+        for (int run = 2; run <= size; run <<= 1)
+            for (int stride = run >> 1; stride > 0; stride >>= 1) {
+                for (int p = threadIdx.x; p < size / 2; p += TB) {
+                    const int t = 2 * p - (p & (stride - 1)), u = t + stride;
+                    const int a = k[t], b = k[u];
+                    if ((a > b) == ((t & run) == 0) && a != b) {
+                        k[t] = b;
+                        k[u] = a;
+                        const double x = v[t];
+                        v[t] = v[u];
+                        v[u] = x;
+                    }
+                }
+                __syncthreads();
+            }
+        for (int t = threadIdx.x; t < m; t += TB) {
+            if (n <= EMIT_CHUNK) {
+                cci[o + t] = k[t];
+                cv[o + t] = v[t];
+            } else {
+                keys[t0 + c0 + t] = k[t];
+                vals[t0 + c0 + t] = v[t];
+            }
+        }
+        __syncthreads();
+    }
+    if (n <= EMIT_CHUNK) return;
+    for (int e = threadIdx.x; e < n; e += TB) {
+        const int key = keys[t0 + e], own = e / EMIT_CHUNK;
+        int r = e - own * EMIT_CHUNK;
+        for (int c = 0; c * EMIT_CHUNK < n; ++c) {
+            if (c == own) continue;
+            const int* q = keys + t0 + c * EMIT_CHUNK;
+            int lo = 0, hi = min(EMIT_CHUNK, n - c * EMIT_CHUNK);
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (q[mid] < key) lo = mid + 1;
+                else hi = mid;
+            }
+            r += lo;
         }
         cci[o + r] = key;
-        cv[o + r] = vals[t];
+        cv[o + r] = vals[t0 + e];
     }
 }
 
