@@ -869,14 +869,13 @@ inline int block_rows(const Sell<T, V>& S) { return bk(S.k); }
 
 // Runs the statement with compile-time KK (warps per slice; for one warp per
 // slice 1, -1, -2 or 0 by the widest slice, see for_rows) and RR (slices per
-// warp for KK <= 1, where one slice of at most two entries is no warp's work
-// by itself; loads in flight per lane for KK > 1) of operator S.
+// warp for KK <= 1; loads in flight per lane for KK > 1) of operator S.
 #define WITH_KR(S, ...)                                                         \
     do {                                                                        \
         if ((S).k == 1 && (S).mw <= 1) {                                        \
             constexpr int KK = -1;                                              \
             switch ((S).r) {                                                    \
-                case 1: { constexpr int RR = 2; __VA_ARGS__; } break;           \
+                case 1: { constexpr int RR = 1; __VA_ARGS__; } break;           \
                 case 2: { constexpr int RR = 2; __VA_ARGS__; } break;           \
                 case 4: { constexpr int RR = 4; __VA_ARGS__; } break;           \
                 default: fail(AIRG_ERR_STATE, "bad slices-per-warp");           \
@@ -884,7 +883,7 @@ inline int block_rows(const Sell<T, V>& S) { return bk(S.k); }
         } else if ((S).k == 1 && (S).mw <= 2) {                                 \
             constexpr int KK = -2;                                              \
             switch ((S).r) {                                                    \
-                case 1: { constexpr int RR = 2; __VA_ARGS__; } break;           \
+                case 1: { constexpr int RR = 1; __VA_ARGS__; } break;           \
                 case 2: { constexpr int RR = 2; __VA_ARGS__; } break;           \
                 case 4: { constexpr int RR = 4; __VA_ARGS__; } break;           \
                 default: fail(AIRG_ERR_STATE, "bad slices-per-warp");           \
@@ -1641,10 +1640,13 @@ long long sell_bytes(const Sell<double>& S, int vbytes)
 // per warp r = 1, 2, 4 for short rows (one warp per slice), loads in flight
 // per lane r = 4, 8, 16 for long rows (several warps per slice), each with
 // the operator's own grid or a resident grid striding over the slices
-// (persist; it removes the partly idle last wave).  None of them changes
-// the arithmetic.  forced > 0 (AIRG_ROWS_PER_WARP for short rows,
-// AIRG_LOADS_PER_LANE for long rows) fixes r, AIRG_PERSIST_GRID=0|1 the
-// grid; with both fixed nothing is timed.
+// (persist; it removes the partly idle last wave).  One slice of at most two
+// entries is too little work for a warp, so r = 1 is not timed there (4096^2,
+// smoother term of level 0 with r = 1, 2, 4: 31.4, 27.1, 28.5 us FP32, 51.3,
+// 49.9, 54.1 us FP64; its residual 49.9, 45.6, 46.2 and 83.0, 82.3, 79.0).
+// None of them changes the arithmetic.  forced > 0 (AIRG_ROWS_PER_WARP for
+// short rows, AIRG_LOADS_PER_LANE for long rows) fixes r, AIRG_PERSIST_GRID=0|1
+// the grid; with both fixed nothing is timed.
 // Returns the time of 3 launches of the chosen variant (0 when not timed).
 template <class T, class V>
 float tune_rows(Sell<T, V>& A, const T* x, T* y, int forced_short, int forced_long, cudaStream_t st)
@@ -1663,6 +1665,7 @@ float tune_rows(Sell<T, V>& A, const T* x, T* y, int forced_short, int forced_lo
     CK(cudaEventCreate(&e1));
     float best = 0.f;
     int best_r = A.k == 1 ? 1 : 4, best_p = 0;
+    const bool narrow = A.k == 1 && A.mw <= 2;
     const int cand_short[3] = {1, 2, 4}, cand_long[3] = {4, 8, 16};
     const int* cand = A.k == 1 ? cand_short : cand_long;
     bool first = true;
@@ -1670,6 +1673,7 @@ float tune_rows(Sell<T, V>& A, const T* x, T* y, int forced_short, int forced_lo
         A.r = forced ? forced : cand[ci % 3];
         A.persist = ci / 3;
         if ((forced && ci % 3) || (forced_p >= 0 && A.persist != forced_p)) continue;
+        if (!forced && narrow && A.r == 1) continue;
         SellView<T, V> v = view(A);
         auto launch = [&]() {
             WITH_KR_COL(A, k_spmv<T, KK, RR, V, C16><<<grid_rows(A, k_spmv<T, KK, RR, V, C16>), block_rows(A), 0, st>>>(v, x, y));
