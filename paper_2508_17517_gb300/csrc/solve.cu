@@ -130,14 +130,20 @@ __global__ void k_sell_pad(int nslices, const int* __restrict__ sptr, int* col)
         if (col[b + 32 * k] < 0) col[b + 32 * k] = m;
 }
 
+int coarse_stream_mode()
+{
+    const char* e = getenv("AIRG_COARSE_STREAM");
+    return e ? atoi(e) : 0;
+}
+
 template <class T>
 void build_sell(const DevCSR& A, const int* src_row, const int* cmap, int n_cols, Sell<T>& S,
-                bool split_diag, cudaStream_t st)
+                bool split_diag, cudaStream_t st, bool fewer_warps = true)
 {
     S.n_rows = A.n_rows;
     S.n_cols = n_cols;
     S.nnz = A.nnz;
-    S.k = choose_parts(A.nnz, A.n_rows, true);
+    S.k = choose_parts(A.nnz, A.n_rows, fewer_warps);
     S.pw = A.n_rows && A.nnz > 12LL * A.n_rows ? 4 : 1;
     S.r = S.k == 1 ? 1 : 4;
     S.n_slices = (A.n_rows + 31) / 32;
@@ -1778,17 +1784,18 @@ void tune_coarse_xs(Sell<T>& A, float unstaged_ms, const T* x, T* y, cudaStream_
 }
 
 // Streamed form of the coarsest operator's steps (coarse_stream.cu),
-// opt-in: AIRG_COARSE_STREAM=1 uses it whenever the layout allows, =2 only
-// where it times faster than the best row-kernel form (`unstaged_ms` for 3
-// launches of y = A x).  Off by default: on the 4096^2 workload its step
-// measured 37.3 against 35.0 us (FP32) and 86.5 against 56.5 us (FP64).
-// Neither form changes the arithmetic.
+// opt-in: AIRG_COARSE_STREAM=1 uses it whenever the layout allows (8 warps
+// per slice, at most 65536 rows), =2 only where it times faster than the best
+// row-kernel form of those 8 warps (`unstaged_ms` for 3 launches of y = A x).
+// Off by default: on the 4096^2 workload, with an earlier hierarchy whose
+// coarsest level had fewer than 65536 rows, its step measured 37.3 against
+// 35.0 us (FP32) and 86.5 against 56.5 us (FP64, 8 warps).  Neither form
+// changes the arithmetic.
 template <class T>
 void tune_coarse_stream(Sell<T>& A, float unstaged_ms, const T* x, T* y, cudaStream_t st)
 {
     A.stream = 0;
-    const char* env = getenv("AIRG_COARSE_STREAM");
-    const int mode = env ? atoi(env) : 0;
+    const int mode = coarse_stream_mode();
     if (mode == 0 || A.xs || !coarse_stream_ok(A)) return;
     if (mode == 1) {
         A.stream = 1;
@@ -2030,7 +2037,9 @@ void build_solve_data(Hierarchy& H, cudaStream_t st)
         CK(cudaStreamSynchronize(st));
         S->lv.push_back(std::move(sl));
     }
-    build_sell<double>(H.coarse.A, iperm[L].p, perm[L].p, S->n_coarse, S->Ac, true, st);
+    // the streamed form shares its arithmetic with 8 warps a slice, so the rule
+    // that gives large FP64 operators fewer stays off where it is asked for
+    build_sell<double>(H.coarse.A, iperm[L].p, perm[L].p, S->n_coarse, S->Ac, true, st, coarse_stream_mode() == 0);
     if (mixed_precision(H.opt)) copy_sell_f32(S->Ac, S->Ac32, st);
     add_col16(S->Ac, st);
     add_col16(S->Ac32, st);
