@@ -3,12 +3,12 @@
 // iterations advanced in lockstep.
 //
 // Layout: a batch of k vectors of length n is stored row-major, [row][rhs],
-// in the nested F/C order of the single solve.  Every operator kernel runs
-// one warp per row with the lanes over right-hand sides (q = lane + 32 j,
-// j < KW): each stored entry of the row is read once per warp (broadcast)
-// and reused for all k right-hand sides, and the gathers of x read k
-// consecutive values of one row -- contiguous, coalesced.  The operator
-// bytes of a V-cycle are thus paid once per k right-hand sides.
+// in the nested F/C order of the single solve.  Every operator kernel gives
+// a row to a group of lanes, each with adjacent right-hand sides (Lanes
+// below): each stored entry of the row is read once per group (broadcast) and
+// reused for all k right-hand sides, and the gathers of x read k consecutive
+// values of one row -- contiguous, coalesced.  The operator bytes of a
+// V-cycle are thus paid once per k right-hand sides.
 //
 // A right-hand side whose FGMRES residual reaches its tolerance is frozen:
 // its next basis vector is zero and its least-squares solution uses only
@@ -383,7 +383,6 @@ __global__ void kb_d2f(long long m, const double* a, float* b)
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < m) b[i] = (float)a[i];
 }
-// [q][i] (caller, natural order) <-> [pos(i)][q] (batch, nested order)
 // [q][i] (caller: right-hand sides one after the other, natural order) <->
 // [pos(i)][q] (batch: rows in nested order, right-hand sides adjacent), a
 // transpose with a row permutation.  A block moves a tile of 32 rows x 32

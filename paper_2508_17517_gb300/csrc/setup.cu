@@ -547,7 +547,8 @@ __global__ void k_scale(int nnz, double* v, double s)
 //     registers;
 //   more: a warp adds them into a hash table in shared memory and ranks the
 //     columns with a bitmap over their range.
-//   rows with more distinct columns than GEMM_CAP: tables in global memory.
+//   rows with more distinct columns than GEMM_CAP: tables in global memory,
+//     sorted by column in shared memory.
 // The sorted rows go to a scratch piece and from there, packed, into C.
 // Bound: latency of the loads of B's rows and of the shared-memory table, at
 // 12-16 warps per SM.  Tables in global memory for every row, sized at twice
@@ -563,19 +564,17 @@ constexpr int GEMM_WARPS = 4;                   // rows per block
 
 __device__ __forceinline__ unsigned hash_col(int j) { return (unsigned)j * 2654435761u; }
 
-// Products of row row0 + li (saturated), the scratch entries of the row
-// (never more than its products or GEMM_CAP), and the row's class list.
-// lists: four of m entries each, counts: their lengths.
-__global__ void k_gemm_bound(int m, int row0, const int* arp, const int* aci, const int* brp, int* prod, int* room)
+// Products of each row (saturated at 2^30 - 1), and its scratch entries: never
+// more than its products or GEMM_CAP.
+__global__ void k_gemm_bound(int m, const int* arp, const int* aci, const int* brp, int* prod, int* room)
 {
-    int li = blockIdx.x * blockDim.x + threadIdx.x;
-    if (li >= m) return;
-    const int i = row0 + li;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m) return;
     long long b = 0;
     for (int p = arp[i]; p < arp[i + 1]; ++p) b += brp[aci[p] + 1] - brp[aci[p]];
     const int n = int(b < 0x3fffffffLL ? b : 0x3fffffffLL);
-    prod[li] = n;
-    room[li] = n < GEMM_CAP ? n : GEMM_CAP;
+    prod[i] = n;
+    room[i] = n < GEMM_CAP ? n : GEMM_CAP;
 }
 
 __device__ __forceinline__ int gemm_class(int b)
@@ -585,7 +584,7 @@ __device__ __forceinline__ int gemm_class(int b)
 
 // Class lists of the rows of a piece (one aggregated atomic per warp and
 // class; the order of a list does not matter), and zero counts for the rows
-// without products.
+// without products.  lists: four of m entries each, counts: their lengths.
 __global__ void k_gemm_lists(int m, const int* prod, int* lists, int* counts, int* cnt)
 {
     const int li = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
@@ -1600,7 +1599,7 @@ void spgemm(const DevCSR& A, const DevCSR& B, DevCSR& C, cudaStream_t st)
     DBuf<unsigned long long> sum(1);
     CK(cudaMemsetAsync(sum.p, 0, sizeof(unsigned long long), st));
     if (m) {
-        k_gemm_bound<<<grid_for(m, TB), TB, 0, st>>>(m, 0, A.rp.p, A.ci.p, B.rp.p, prod.p, room.p);
+        k_gemm_bound<<<grid_for(m, TB), TB, 0, st>>>(m, A.rp.p, A.ci.p, B.rp.p, prod.p, room.p);
         k_sum_int<<<std::min(grid_for(m, TB), 1024), TB, 0, st>>>(m, room.p, sum.p);
     }
     CK_LAUNCH();

@@ -77,7 +77,7 @@ struct Sell {
 
 template <class T, class V = T>
 struct SellView {
-    int n_rows, n_slices, mw;
+    int n_rows, n_slices;
     const int* __restrict__ sptr;
     const int* __restrict__ col;
     const V* __restrict__ val;
@@ -89,7 +89,7 @@ struct SellView {
 template <class T, class V>
 SellView<T, V> view(const Sell<T, V>& s)
 {
-    return SellView<T, V>{s.n_rows, s.n_slices, s.mw, s.sptr.p, s.col.p, s.val.p, s.ndiag ? s.diag.p : nullptr,
+    return SellView<T, V>{s.n_rows, s.n_slices, s.sptr.p, s.col.p, s.val.p, s.ndiag ? s.diag.p : nullptr,
                           s.col16.n ? s.col16.p : nullptr, s.cbase.n ? s.cbase.p : nullptr};
 }
 
