@@ -533,9 +533,9 @@ __device__ __forceinline__ void dot_slices(const SellView<T, V>& S, const X* __r
 // Applies epi(r, (S x)_r, pre(r)) to every row r of S.  pre(r) loads the
 // row's other operands; it runs before the row's gathers so that its loads
 // overlap them.  K = warps per slice; for one warp per slice K is -1 or -2 (no
-// slice wider than one, two entries), 1 (four on average) or 0 (more).  R = slices per warp for K = 1, and
-// loads in flight per lane (4, 8 or 16) for K > 1; in neither case does R
-// change the arithmetic.
+// slice wider than one, two entries), 1 (four on average) or 0 (more).  R =
+// slices per warp for K <= 1, and loads in flight per lane (4, 8 or 16) for
+// K > 1; in neither case does R change the arithmetic.
 template <class T, int K, int R, bool C16 = false, class V, class X, class Pre, class Epi>
 __device__ __forceinline__ void for_rows(const SellView<T, V>& S, const X* __restrict__ x, const Pre& pre,
                                          const Epi& epi, int rev = 0)

@@ -161,15 +161,19 @@ inline int parts_for(double avg, int per_lane, int max_parts)
 // warps) give the shortest chains.  In FP64, operators with enough slices to
 // fill the GPU take fewer, because each further warp per slice adds its
 // partial sums to the row (four per warp: with 8, 31 additions on top of a
-// row of 66 products, in the FP64 pipe).  The line, 2800 warps (18 per SM)
-// and at most 48 entries per lane, measured: residual of 70,639 rows of 66
-// entries with 8, 4, 2 warps 32.0, 28.2, 23.6 us; 42,872 rows of 86 with 8,
-// 4, 2: 25.7, 21.1, 25.6 us; smoother term of 117,848 rows of 28 with 4, 2,
+// row of 66 products, in the FP64 pipe).  The line, 2800 warps (18 on each of
+// 152 SMs) and at most 48 entries per lane, measured: residual of 70,639 rows
+// of 66 entries with 8, 4, 2 warps 32.0, 28.2, 23.6 us; 42,872 rows of 86 with
+// 8, 4, 2: 25.7, 21.1, 25.6 us; smoother term of 117,848 rows of 28 with 4, 2,
 // 1: 23.4, 19.2, 18.1 us; coarse step of 105,946 rows of 67 with 8, 4, 2:
 // 33.5, 29.9, 28.3 us; residual of 17,911 rows of 61 with 8, 4, 2: 13.9,
-// 15.0, 19.9 us.  In FP32, where additions are free, the line gains nothing
-// on average and loses on the longest rows (80,178 of 163: 24.0 -> 27.2 us).
-// AIRG_MAX_PARTS / AIRG_PER_LANE set the cap and the 12, without the line.
+// 15.0, 19.9 us.  These put it between 2,680 warps (too few) and 3,683
+// (enough); where in between is open.  In FP32, where additions are free, the
+// line gains nothing on average and loses on the longest rows (80,178 of 163:
+// 24.0 -> 27.2 us).  It is a number and not a multiple of the SM count because
+// the warps fix the order of a row's sum, and with it the result.
+// AIRG_MAX_PARTS / AIRG_PER_LANE set the cap and the 12, without the line;
+// AIRG_COARSE_STREAM does without it for the coarsest operator.
 inline int choose_parts(long long nnz, int n_rows, bool fp64)
 {
     const char* e = getenv("AIRG_MAX_PARTS");
