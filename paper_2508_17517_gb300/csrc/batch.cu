@@ -50,7 +50,8 @@ template <class T, int VEC, int KW>
 struct Lanes {
     int ql, lg, k;
     __device__ __forceinline__ int q(int j) const { return (ql + (j << lg)) * VEC; }
-    __device__ __forceinline__ bool ok(int j) const { return q(j) < k; }
+    // KW = 2 and 4 hold more than 32 and 64 packs
+    __device__ __forceinline__ bool ok(int j) const { return j < KW / 2 || q(j) < k; }
 };
 template <class T, int VEC>
 struct alignas(sizeof(T) * VEC) Pack {
@@ -82,16 +83,24 @@ __device__ __forceinline__ void bstore(const Lanes<T, VEC, KW>& L, T* a, long lo
     for (int j = 0; j < KW; ++j)
         if (L.ok(j)) *reinterpret_cast<Pack<T, VEC>*>(a + size_t(r) * L.k + L.q(j)) = o.p[j];
 }
-// o = f(values of the operands), element by element
+// a[r] = f(values of the operands), element by element.  With four steps of
+// the warp the values are formed under the store's condition, so that a step
+// past the last right-hand side costs no FP64 work (96 right-hand sides, FP64,
+// 1024^2: 244.9 -> 241.6 ms); with fewer, all steps but the last are full and
+// that condition costs registers (31: 78.5 -> 80.0 ms).
 template <class T, int VEC, int KW, class F, class... A>
-__device__ __forceinline__ Vals<T, VEC, KW> beach(const F& f, const Vals<T, VEC, KW>& a, const A&... more)
+__device__ __forceinline__ void bstore(const Lanes<T, VEC, KW>& L, T* a, long long r, const F& f,
+                                       const Vals<T, VEC, KW>& x, const A&... more)
 {
     Vals<T, VEC, KW> o;
 #pragma unroll
-    for (int j = 0; j < KW; ++j)
+    for (int j = 0; j < KW; ++j) {
+        if (KW == 4 && !L.ok(j)) continue;
 #pragma unroll
-        for (int u = 0; u < VEC; ++u) o.p[j].v[u] = f(a.p[j].v[u], more.p[j].v[u]...);
-    return o;
+        for (int u = 0; u < VEC; ++u) o.p[j].v[u] = f(x.p[j].v[u], more.p[j].v[u]...);
+        if (KW == 4) *reinterpret_cast<Pack<T, VEC>*>(a + size_t(r) * L.k + L.q(j)) = o.p[j];
+    }
+    if (KW < 4) bstore(L, a, r, o);
 }
 
 // Rows of operator S times the k right-hand sides x ([row][rhs]): row r is
@@ -103,8 +112,14 @@ __device__ __forceinline__ Vals<T, VEC, KW> beach(const F& f, const Vals<T, VEC,
 // not depend on timing.  pre(r, L) loads the row's other operands before the
 // product, so those loads overlap the gathers; entries are taken four at a
 // time with all their loads issued before their FMAs, which run in entry
-// order.  Then epi(r, L, sums, pre) runs once per row.  `dot` = false skips
-// the product (sums 0).  Every thread of the block reaches the barrier.
+// order, and up to three that are left together too.  Rows of several steps
+// of a warp (KW > 1) take those one by one, know their row's warp at compile
+// time and add zeros for lanes without a right-hand side: each of these saves
+// registers, and with them a third of the warps in flight (FP64, 1024^2: 33
+// right-hand sides 137 -> 122 ms, 65 300 -> 237, 127 327 -> 253; FP32: 63 59
+// -> 55, 65 94 -> 69, 127 114 -> 88).  Then epi(r, L, sums, pre) runs once per
+// row.  `dot` = false skips the product (sums 0).  Every thread of the block
+// reaches the barrier.
 // X: the type x is stored in (FP32 under an FP64 operator: widened exactly).
 template <class T, int VEC, int KW, int PW, class V, class X, class Pre, class Epi>
 __device__ __forceinline__ void bfor_rows(const SellView<T, V>& S, const X* __restrict__ x, int k, int lg,
@@ -115,10 +130,12 @@ __device__ __forceinline__ void bfor_rows(const SellView<T, V>& S, const X* __re
     using PV = decltype(pre(0, LN{}));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int part = warp % PW;
+    if constexpr (KW > 1) lg = 5;   // a whole warp a row
     const LN L{lane & ((1 << lg) - 1), lg, k};
     // rev != 0: blocks take the rows in reverse order (serpentine chains)
     const int bx = rev ? int(gridDim.x) - 1 - int(blockIdx.x) : int(blockIdx.x);
-    const long long rr = ((long long)bx * (BT / 32 / PW) + warp / PW) * (32 >> lg) + (lane >> lg);
+    long long rr = (long long)bx * (BT / 32 / PW) + warp / PW;
+    if constexpr (KW == 1) rr = rr * (32 >> lg) + (lane >> lg);
     const bool valid = rr < S.n_rows;
     const int r = valid ? int(rr) : 0;
     const bool lead = valid && part == 0;
@@ -157,15 +174,31 @@ __device__ __forceinline__ void bfor_rows(const SellView<T, V>& S, const X* __re
 #pragma unroll
                 for (int j = 0; j < KW; ++j)
                     if (L.ok(j)) xv[u][j] = *reinterpret_cast<const PK*>(xr[u] + L.q(j));
+                    else if constexpr (VEC == 1)
+#pragma unroll
+                        for (int i = 0; i < VEC; ++i) xv[u][j].v[i] = X(0);
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
                 for (int j = 0; j < KW; ++j)
-                    if (L.ok(j))
+                    if (VEC == 1 || L.ok(j))
 #pragma unroll
                         for (int i = 0; i < VEC; ++i) acc.p[j].v[i] = fma(v[u], wide<T>(xv[u][j].v[i]), acc.p[j].v[i]);
         }
-        if (e < w) {   // up to three entries left, their loads together too
+        if constexpr (KW > 1) {
+            for (; e < w; e += PW) {
+                const int idx = b + 32 * e;
+                const T v = ldval<T>(S.val + idx);
+                const X* xr = x + size_t(__ldg(S.col + idx)) * k;
+#pragma unroll
+                for (int j = 0; j < KW; ++j)
+                    if (L.ok(j)) {
+                        const PK xv = *reinterpret_cast<const PK*>(xr + L.q(j));
+#pragma unroll
+                        for (int i = 0; i < VEC; ++i) acc.p[j].v[i] = fma(v, wide<T>(xv.v[i]), acc.p[j].v[i]);
+                    }
+            }
+        } else if (e < w) {   // up to three entries left, their loads together too
             T v[3];
             const X* xr[3];
             PK xv[3][KW];
@@ -238,7 +271,7 @@ __global__ void kb_restrict(SellView<T, V> Z, const T* __restrict__ sf, const T*
     using VL = Vals<T, VEC, KW>;
     bfor_rows<T, VEC, KW, PW>(Z, sf, k, lg, true, [&](int r, const LN& L) { return bload(L, sc, r); },
                               [&](int r, const LN& L, const VL& d, const VL& c) {
-                                  bstore(L, dc, r, beach<T, VEC, KW>([](T a, T b) { return a + b; }, c, d));
+                                  bstore(L, dc, r, [](T a, T b) { return a + b; }, c, d);
                               });
 }
 
@@ -250,9 +283,8 @@ __global__ void kb_fresid(SellView<T> M, const T* __restrict__ rf, const T* __re
     using VL = Vals<T, VEC, KW>;
     bfor_rows<T, VEC, KW, PW>(M, ec, k, lg, true, [&](int r, const LN& L) { return bload(L, rf, r); },
                               [&](int r, const LN& L, const VL& d, const VL& f) {
-                                  const VL tt = beach<T, VEC, KW>([](T a, T b) { return a - b; }, f, d);
-                                  bstore(L, t, r, tt);
-                                  bstore(L, w, r, beach<T, VEC, KW>([&](T a) { return ap * a; }, tt));
+                                  bstore(L, t, r, [](T a, T b) { return a - b; }, f, d);
+                                  bstore(L, w, r, [&](T a, T b) { return ap * (a - b); }, f, d);
                               });
 }
 
@@ -264,7 +296,7 @@ __global__ void kb_horner(SellView<T> A, const T* __restrict__ t, const T* __res
     using VL = Vals<T, VEC, KW>;
     bfor_rows<T, VEC, KW, PW>(A, win, k, lg, true, [&](int r, const LN& L) { return bload(L, t, r); },
                               [&](int r, const LN& L, const VL& d, const VL& tv) {
-                                  bstore(L, wout, r, beach<T, VEC, KW>([&](T a, T b) { return fma(ak, a, b); }, tv, d));
+                                  bstore(L, wout, r, [&](T a, T b) { return fma(ak, a, b); }, tv, d);
                               }, rev);
 }
 
@@ -279,8 +311,7 @@ __global__ void kb_horner_last(SellView<T> A, const T* __restrict__ t, const T* 
     bfor_rows<T, VEC, KW, PW>(A, win, k, lg, true,
                               [&](int r, const LN& L) { return V2{bload(L, t, r), bload(L, ec, W[r])}; },
                               [&](int r, const LN& L, const VL& d, const V2& q) {
-                                  bstore(L, ef, r, beach<T, VEC, KW>([&](T e, T a, T b) { return e + fma(a0, a, b); },
-                                                                     q.b, q.a, d));
+                                  bstore(L, ef, r, [&](T e, T a, T b) { return e + fma(a0, a, b); }, q.b, q.a, d);
                               }, rev);
 }
 
@@ -297,8 +328,7 @@ __global__ void kb_horner_acc(SellView<T> A, const T* __restrict__ t, const T* _
     bfor_rows<T, VEC, KW, PW>(A, win, k, lg, true,
                               [&](int r, const LN& L) { return V2{bload(L, t, r), bload(L, (const T*)e, r)}; },
                               [&](int r, const LN& L, const VL& d, const V2& q) {
-                                  bstore(L, e, r, beach<T, VEC, KW>([&](T ee, T a, T b) { return ee + fma(a0, a, b); },
-                                                                    q.b, q.a, d));
+                                  bstore(L, e, r, [&](T ee, T a, T b) { return ee + fma(a0, a, b); }, q.b, q.a, d);
                               }, rev);
 }
 
@@ -341,10 +371,9 @@ __global__ void kb_newton_real(SellView<T> A, const T* __restrict__ rin, T* __re
                                   return V2{bload(L, rin, r), bload(L, first ? (const T*)nullptr : (const T*)x, r)};
                               },
                               [&](int r, const LN& L, const VL& d, const V2& q) {
-                                  bstore(L, x, r, beach<T, VEC, KW>([&](T a, T b) { return fma(a, inv, b); }, q.a, q.b));
+                                  bstore(L, x, r, [&](T a, T b) { return fma(a, inv, b); }, q.a, q.b);
                                   if (!last)
-                                      bstore(L, rout, r,
-                                             beach<T, VEC, KW>([&](T a, T b) { return a - b * inv; }, q.a, d));
+                                      bstore(L, rout, r, [&](T a, T b) { return a - b * inv; }, q.a, d);
                               }, rev);
 }
 
@@ -360,9 +389,8 @@ __global__ void kb_newton_pair1(SellView<T> A, const T* __restrict__ rin, T* __r
                                   return V2{bload(L, rin, r), bload(L, first ? (const T*)nullptr : (const T*)x, r)};
                               },
                               [&](int r, const LN& L, const VL& d, const V2& q) {
-                                  const VL tt = beach<T, VEC, KW>([&](T a, T b) { return two_a * a - b; }, q.a, d);
-                                  bstore(L, t, r, tt);
-                                  bstore(L, x, r, beach<T, VEC, KW>([&](T a, T b) { return fma(a, inv2, b); }, tt, q.b));
+                                  bstore(L, t, r, [&](T a, T b) { return two_a * a - b; }, q.a, d);
+                                  bstore(L, x, r, [&](T a, T b, T c) { return fma(two_a * a - b, inv2, c); }, q.a, d, q.b);
                               }, rev);
 }
 
@@ -374,7 +402,7 @@ __global__ void kb_newton_pair2(SellView<T> A, const T* __restrict__ rin, const 
     using VL = Vals<T, VEC, KW>;
     bfor_rows<T, VEC, KW, PW>(A, t, k, lg, true, [&](int r, const LN& L) { return bload(L, rin, r); },
                               [&](int r, const LN& L, const VL& d, const VL& ri) {
-                                  bstore(L, rout, r, beach<T, VEC, KW>([&](T a, T b) { return a - b * inv2; }, ri, d));
+                                  bstore(L, rout, r, [&](T a, T b) { return a - b * inv2; }, ri, d);
                               }, rev);
 }
 
@@ -570,25 +598,31 @@ __global__ void kb_sub(long long m, const double* b, const double* y, double* r)
 // Shape of a batch of k vectors of type T (Lanes): 16-byte packs where every
 // row of k values starts on a 16-byte boundary, the smallest power of two of
 // lanes that covers the packs, and KW steps of a whole warp beyond 32.
+// `packs` false: FP64 batches of more than 32 take none.  There the lanes are
+// all used without, and the registers of the packs' loads in flight (56 a
+// thread against 32) cost warps: 64 right-hand sides on 2048^2 602 -> 535 ms,
+// 32 as packs 306.  The top-level product of an FP32 V-cycle's vectors, which
+// reads half the bytes, is faster with them (64 on 2048^2: 18.1 against 25.4
+// ms a solve).
 struct BShape {
     int vec, lg, kw;
 };
 template <class T>
-BShape bshape(int k)
+BShape bshape(int k, bool packs)
 {
     const int full = 16 / int(sizeof(T));
-    BShape s{k % full == 0 ? full : 1, 0, 1};
-    const int packs = k / s.vec;
-    while (s.lg < 5 && (1 << s.lg) < packs) ++s.lg;
-    s.kw = packs <= 32 ? 1 : (packs <= 64 ? 2 : 4);
+    BShape s{k % full == 0 && (packs || sizeof(T) == 4 || k <= 32) ? full : 1, 0, 1};
+    const int n = k / s.vec;
+    while (s.lg < 5 && (1 << s.lg) < n) ++s.lg;
+    s.kw = n <= 32 ? 1 : (n <= 64 ? 2 : 4);
     return s;
 }
 
 // Runs the statement with VEC, KW and lg of a batch of k vectors of type T,
 // and PW (warps per row: 1 for operators with short rows, 4 for long rows)
-// of operator S.  (16-byte packs: at most 128 / 4 FP32 or 128 / 2 FP64
-// lanes, so KW = 1, or 2 in FP64.)
-#define WITH_SHAPE(T, bs, ...)                                                       \
+// of operator S.  PKW: the most steps that packs take (16-byte packs: at most
+// 128 / 4 FP32 or, without `packs`, 32 / 2 FP64 lanes, one step).
+#define WITH_SHAPE(T, PKW, bs, ...)                                                  \
     do {                                                                             \
         if ((bs).vec == 1) {                                                         \
             constexpr int VEC = 1;                                                   \
@@ -598,16 +632,17 @@ BShape bshape(int k)
         } else {                                                                     \
             constexpr int VEC = 16 / int(sizeof(T));                                 \
             if ((bs).kw == 1) { constexpr int KW = 1; __VA_ARGS__; }                 \
-            else { constexpr int KW = sizeof(T) == 8 ? 2 : 1; __VA_ARGS__; }         \
+            else { constexpr int KW = PKW; __VA_ARGS__; }                            \
         }                                                                            \
     } while (0)
-#define WITH_BATCH(T, k, S, ...)                                                     \
+#define WITH_BATCH_SHAPE(T, PKW, bs, S, ...)                                         \
     do {                                                                             \
-        const BShape bs_ = bshape<T>(k);                                             \
+        const BShape bs_ = (bs);                                                     \
         const int lg = bs_.lg;                                                       \
-        if ((S).pw == 1) { constexpr int PW = 1; WITH_SHAPE(T, bs_, __VA_ARGS__); }  \
-        else { constexpr int PW = 4; WITH_SHAPE(T, bs_, __VA_ARGS__); }              \
+        if ((S).pw == 1) { constexpr int PW = 1; WITH_SHAPE(T, PKW, bs_, __VA_ARGS__); } \
+        else { constexpr int PW = 4; WITH_SHAPE(T, PKW, bs_, __VA_ARGS__); }         \
     } while (0)
+#define WITH_BATCH(T, k, S, ...) WITH_BATCH_SHAPE(T, 1, bshape<T>(k, false), S, __VA_ARGS__)
 
 }  // namespace
 
@@ -1044,7 +1079,7 @@ void solve_batched(Hierarchy& H, int k, const double* b, double* x, double rtol,
                 float* zj = B.Zs32.p + size_t(j) * nk;
                 bprecond(H, B, (const float*)B.vin32.p, zj, st);
                 LAUNCH_F(S, PK_TOPSPMV, topB - 4 * nk, 2 * S.Atop.nnz * k,
-                       WITH_BATCH(double, k, S.Atop, kb_spmv<double, VEC, KW, PW, float><<<grid_rows(n, PW, lg), BT, 0, st>>>(A, zj, B.w.p, k, lg)));
+                       WITH_BATCH_SHAPE(double, 2, bshape<double>(k, true), S.Atop, kb_spmv<double, VEC, KW, PW, float><<<grid_rows(n, PW, lg), BT, 0, st>>>(A, zj, B.w.p, k, lg)));
             } else {
                 double* zj = B.Zs.p + size_t(j) * nk;
                 bprecond(H, B, (const double*)vj, zj, st);
