@@ -658,7 +658,6 @@ struct BatchData {
     HBuf<double> hh;
     struct GEntry { const void* v; void* z; cudaGraphExec_t exec; long long kernels; };
     std::vector<GEntry> graphs;
-    std::vector<std::pair<const void*, void*>> seen;   // pairs used before (graph captured at the second use)
     ~BatchData()
     {
         for (GEntry& g : graphs) cudaGraphExecDestroy(g.exec);
@@ -921,34 +920,31 @@ void bprecond(Hierarchy& H, BatchData& B, const T* v, T* z, cudaStream_t st)
     BatchData::GEntry* ge = nullptr;
     for (auto& g : B.graphs)
         if (g.v == v && g.z == z) { ge = &g; break; }
-    if (!ge && first_use(B.seen, v, z)) {
-        bprecond_launch(H, B, v, z, st);
+    if (ge) {
+        CK(cudaGraphLaunch(ge->exec, st));
+        S.launches += ge->kernels;
         return;
     }
-    if (!ge) {
-        long long before = S.launches;
-        CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        try {
-            bprecond_launch(H, B, v, z, st);
-        } catch (...) {
-            cudaGraph_t g0;
-            cudaStreamEndCapture(st, &g0);
-            if (g0) cudaGraphDestroy(g0);
-            throw;
-        }
-        cudaGraph_t graph;
-        CK(cudaStreamEndCapture(st, &graph));
-        cudaGraphExec_t exec;
-        cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
-        cudaGraphDestroy(graph);
-        CK(e);
-        long long nkern = S.launches - before;
-        S.launches = before;
-        B.graphs.push_back(BatchData::GEntry{v, z, exec, nkern});
-        ge = &B.graphs.back();
+    // first use: launched directly, and captured while the kernels run
+    bprecond_launch(H, B, v, z, st);
+    const long long before = S.launches;
+    CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+    try {
+        bprecond_launch(H, B, v, z, st);
+    } catch (...) {
+        cudaGraph_t g0;
+        cudaStreamEndCapture(st, &g0);
+        if (g0) cudaGraphDestroy(g0);
+        throw;
     }
-    CK(cudaGraphLaunch(ge->exec, st));
-    S.launches += ge->kernels;
+    cudaGraph_t graph;
+    CK(cudaStreamEndCapture(st, &graph));
+    cudaGraphExec_t exec;
+    cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
+    cudaGraphDestroy(graph);
+    CK(e);
+    B.graphs.push_back(BatchData::GEntry{v, z, exec, S.launches - before});
+    S.launches = before;
 }
 
 void ensure_batch(Hierarchy& H, int k)

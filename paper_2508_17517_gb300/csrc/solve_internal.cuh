@@ -9,7 +9,6 @@
 #include <cstdlib>
 #include <memory>
 #include <string>
-#include <utility>
 #include <vector>
 
 #include "dev_util.cuh"
@@ -371,7 +370,6 @@ struct SolveData {
     bool use_graphs = true;
     struct GEntry { const void* v; void* z; cudaGraphExec_t exec; long long kernels; };
     std::vector<GEntry> graphs;
-    std::vector<std::pair<const void*, void*>> seen;   // pairs used before (graph captured at the second use)
     ~SolveData()
     {
         for (cudaEvent_t e : evpool) cudaEventDestroy(e);
@@ -381,17 +379,6 @@ struct SolveData {
         if (sst) cudaStreamDestroy(sst);
     }
 };
-
-// True, and noted, the first time this (input, output) pair of the handle's
-// own vectors is preconditioned.
-inline bool first_use(std::vector<std::pair<const void*, void*>>& seen, const void* v, void* z)
-{
-    const std::pair<const void*, void*> p(v, z);
-    for (const auto& q : seen)
-        if (q == p) return false;
-    seen.push_back(p);
-    return true;
-}
 
 // Runs the statement with the compile-time constant MM = mv (1..16).
 #define WITH_M(mv, ...)                                                         \
