@@ -27,7 +27,7 @@ def test_second_solve_replays(prec, nrhs):
     shape = (256 * 256,) if nrhs == 1 else (nrhs, 256 * 256)
     b = torch.randn(*shape, dtype=torch.float64, device="cuda", generator=gen)
     second, later = [], []
-    for _ in range(7):
+    for _ in range(15):
         h = G.airg_setup(pg["rowptr"], pg["col"], pg["val"],
                          G.airg_options_default(**dict(w["opts"], precision=prec)))
         ms, xs, launches = [], [], []
